@@ -43,6 +43,24 @@ template <> struct Store<__nv_bfloat16> {
 // ReLU with a canonical +0 for every non-positive input.
 __device__ __forceinline__ float relu_f(float v) { return v > 0.f ? v : 0.f; }
 
+// ascending unsigned order of the result == descending float order; -0 -> +0
+__device__ __forceinline__ uint32_t ord_desc(float f) {
+  f = f + 0.0f;
+  const uint32_t u = __float_as_uint(f);
+  const uint32_t asc = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return ~asc;
+}
+
+// Count `key` (if `keep`) in the top-12-bit histogram: the lanes of a warp
+// that share a bin add their count with one atomic (valid logits crowd into
+// a few dozen bins, so per-key atomics would serialise on them).  Every lane
+// of the warp must call it.
+__device__ __forceinline__ void hist_add(uint32_t* hist0, bool keep, uint32_t key, int lane) {
+  const uint32_t bin = keep ? (key >> 20) : 0xFFFFFFFFu;
+  const unsigned peers = __match_any_sync(0xFFFFFFFFu, bin);
+  if (keep && lane == __ffs(peers) - 1) atomicAdd(&hist0[bin], (uint32_t)__popc(peers));
+}
+
 // Device error flag bits (OR-ed into the context's error word).
 enum : int {
   ERR_WAIT_PRODUCER = 1,

@@ -98,9 +98,13 @@ struct rtcc_ctx {
   // RTCC_FLAG_MULTISCALE: the branches end at their blocks; the post-join
   // fuses each block's map across the agents, then runs the neck once
   bool ms = false;
+  // Max fusion or multi-scale: the post-join runs the neck, the max and the
+  // head in one kernel over the blocks' outputs (neck_head.cu), and the
+  // feature maps are computed only when they are read back
+  bool fused_neck = false;
   void* fblk[RTCC_MAX_BLOCKS] = {};   // fused block maps [H_b][W_b][C_b]
   void* neck_out = nullptr;           // neck of the fused blocks [H'][W'][C_feat]
-  std::vector<ConvLayer> neck_layers; // its deconvs (one "agent")
+  std::vector<ConvLayer> neck_layers; // the deconvs, when they are not layers of the branches
   BackboneParams* neck_p = nullptr;
   unsigned* neck_bar = nullptr;       // [kMaxLayers + 1], zero between launches
   int* d_one = nullptr;               // [RTCC_MAX_AGENTS] = {1, 0, ...}: the head's one input
@@ -555,63 +559,42 @@ rtcc_status build_backbone(rtcc_ctx* c) {
       RS(dalloc(c, &c->fblk[bi], (size_t)c->block_w[bi] * c->block_h[bi] * g.block_ch[bi] * es));
     RS(dalloc(c, &c->neck_out, c->feat_elems * es));
     CK(cudaMemset(c->neck_out, 0, c->feat_elems * es));
-    for (int bi = 0; bi < g.n_blocks; ++bi) {
-      ConvLayer L{};
-      L.kind = DECONV;
-      L.n_agents = 1;
-      L.s = g.up_stride[bi];
-      L.cin = g.block_ch[bi];
-      L.cout = g.up_ch;
-      L.in_w = c->block_w[bi];
-      L.in_h = c->block_h[bi];
-      L.out_w = c->Wf;
-      L.out_h = c->Hf;
-      L.gw = L.in_w;
-      L.gh = L.in_h;
-      L.ldc = c->Cf;
-      L.choff = bi * g.up_ch;
-      L.bn = g.up_ch;
-      L.bk = (L.cin >= 64) ? 64 : 32;
-      L.n_tiles_n = L.s * L.s;
-      L.splits = 1;
-      L.in = c->fblk[bi];
-      L.in_astride = (long long)c->block_w[bi] * c->block_h[bi] * g.block_ch[bi];
-      L.out = c->neck_out;
-      L.out_astride = (long long)c->feat_elems;
-      L.wpacked = c->wbufs[wi];
-      L.bias = c->bbufs[wi];
-      L.wait_layers = 0;                              // the fused maps precede the launch
-      ++wi;
+  }
+  c->fused_neck = neck && (c->ms || g.fusion == RTCC_FUSE_MAX) &&
+                  !(g.flags & (RTCC_FLAG_KEEP_FUSED | RTCC_FLAG_LAYER_TIMES)) &&
+                  neck_head_ok(g.n_blocks, g.block_ch, g.up_stride, g.up_ch);
+  const bool apart = c->ms || c->fused_neck;   // the deconvs are not layers of the branches
+  for (int bi = 0; neck && bi < g.n_blocks; ++bi) {
+    ConvLayer L{};
+    L.kind = DECONV;
+    L.n_agents = c->ms ? 1 : K;
+    L.s = g.up_stride[bi];
+    L.cin = g.block_ch[bi];
+    L.cout = g.up_ch;
+    L.in_w = c->block_w[bi];
+    L.in_h = c->block_h[bi];
+    L.out_w = c->Wf;
+    L.out_h = c->Hf;
+    L.gw = L.in_w;
+    L.gh = L.in_h;
+    L.ldc = c->Cf;
+    L.choff = bi * g.up_ch;
+    L.bn = g.up_ch;
+    L.bk = (L.cin >= 64) ? 64 : 32;
+    L.n_tiles_n = L.s * L.s;
+    L.splits = 1;
+    L.in = c->ms ? c->fblk[bi] : c->block_out[bi];
+    L.in_astride = (long long)c->block_w[bi] * c->block_h[bi] * g.block_ch[bi];
+    L.out = c->ms ? c->neck_out : c->feat_all;
+    L.out_astride = (long long)c->feat_elems;
+    L.wpacked = c->wbufs[wi];
+    L.bias = c->bbufs[wi];
+    L.wait_layers = apart ? 0 : block_last[bi];       // only its block's output
+    ++wi;
+    if (apart) {
       if (conv_make_maps(L, c->bf16) != cudaSuccess) return RTCC_E_CUDA;
       c->neck_layers.push_back(L);
-    }
-  } else if (neck) {
-    for (int bi = 0; bi < g.n_blocks; ++bi) {
-      ConvLayer L{};
-      L.kind = DECONV;
-      L.n_agents = K;
-      L.s = g.up_stride[bi];
-      L.cin = g.block_ch[bi];
-      L.cout = g.up_ch;
-      L.in_w = c->block_w[bi];
-      L.in_h = c->block_h[bi];
-      L.out_w = c->Wf;
-      L.out_h = c->Hf;
-      L.gw = L.in_w;
-      L.gh = L.in_h;
-      L.ldc = c->Cf;
-      L.choff = bi * g.up_ch;
-      L.bn = g.up_ch;
-      L.bk = (L.cin >= 64) ? 64 : 32;
-      L.n_tiles_n = L.s * L.s;
-      L.in = c->block_out[bi];
-      L.in_astride = (long long)c->block_w[bi] * c->block_h[bi] * g.block_ch[bi];
-      L.out = c->feat_all;
-      L.out_astride = (long long)c->feat_elems;
-      L.wpacked = c->wbufs[wi];
-      L.bias = c->bbufs[wi];
-      L.wait_layers = block_last[bi];                 // only its block's output
-      ++wi;
+    } else {
       c->layers.push_back(L);
     }
   }
@@ -665,7 +648,7 @@ rtcc_status build_backbone(rtcc_ctx* c) {
   }
   c->launch_p = new (std::nothrow) BackboneParams;
   if (!c->launch_p) return RTCC_E_NOMEM;
-  if (c->ms) {
+  if (apart) {
     RS(dalloc(c, &c->neck_bar, (kMaxLayers + 1) * sizeof(unsigned)));
     CK(cudaMemset(c->neck_bar, 0, (kMaxLayers + 1) * sizeof(unsigned)));
     c->neck_p = new (std::nothrow) BackboneParams;
@@ -860,6 +843,35 @@ rtcc_status capture_post(rtcc_ctx* c) {
     fb.attention = c->cfg.fusion == RTCC_FUSE_ATTN;
     fb.span = c->fuse_span;
   }
+  NeckHeadParams nh{};
+  if (c->fused_neck) {
+    NeckHeadArgs a{};
+    a.n_blocks = c->cfg.n_blocks;
+    for (int bi = 0; bi < a.n_blocks; ++bi) {
+      const ConvLayer& L = c->neck_layers[bi];
+      a.in[bi] = L.in;
+      a.astride[bi] = L.in_astride;
+      a.cin[bi] = L.cin;
+      a.stride[bi] = L.s;
+      a.w[bi] = L.wpacked;
+      a.bias[bi] = L.bias;
+    }
+    a.head_w = c->head_w16;
+    a.feat_w = c->Wf;
+    a.feat_h = c->Hf;
+    a.present = c->ms ? c->d_one : c->d_present;
+    a.K = c->ms ? 1 : c->K;
+    a.head_b = c->head_b;
+    a.head_out = c->head_out;
+    a.keys = c->keys;
+    a.hist0 = c->hist0;
+    a.cls_thresh = c->cfg.cls_thresh;
+    a.anchors = c->cfg.anchors;
+    a.err = c->d_err;
+    a.span = c->ms ? nullptr : c->fuse_span;
+    a.wait_budget = c->wait_budget;
+    CK(neck_head_fill(a, c->bf16, &nh));
+  }
   const bool two_step = c->ms || attn1;
   const int K_head = two_step ? 1 : c->K;
   FuseArgs fa{};
@@ -882,9 +894,9 @@ rtcc_status capture_post(rtcc_ctx* c) {
   // memory, head as an N = 16 MMA); attention fusion: CUDA-core kernel
   const int bkc = fuse_tc_chunk(c->Cf, K_head);
   const bool use_tc = (two_step || !fa.attention) && bkc > 0;
-  if (two_step && !use_tc) return RTCC_E_ARG;
+  if (two_step && !use_tc && !c->fused_neck) return RTCC_E_ARG;
   FuseTcParams tp{};
-  if (use_tc) {
+  if (use_tc && !c->fused_neck) {
     const int swz = bkc * 2;                    // 128- or 64-byte rows
     for (int k = 0; k < K_head; ++k)
       CK(tmap_2d(&tp.feat[k], c->ms ? c->neck_out : (attn1 ? c->fused : c->br[k].feat), c->bf16,
@@ -948,11 +960,15 @@ rtcc_status capture_post(rtcc_ctx* c) {
   if (two_step) {
     if (e == cudaSuccess) e = launch_fuse_blocks(fb, c->bf16, c->post);
     if (e == cudaSuccess && tl) e = record_node(c->ev_fuse1, c->post);
-    if (e == cudaSuccess && c->ms) e = launch_backbone(*c->neck_p, c->bf16, c->post);
-    if (e == cudaSuccess) e = launch_fuse_max_head(tp, c->bf16, c->post);
+    if (e == cudaSuccess && c->ms && !c->fused_neck) e = launch_backbone(*c->neck_p, c->bf16, c->post);
+    if (e == cudaSuccess)
+      e = c->fused_neck ? launch_neck_max_head(nh, c->bf16, c->post)
+                        : launch_fuse_max_head(tp, c->bf16, c->post);
   } else {
     if (e == cudaSuccess) {
-      if (use_tc)
+      if (c->fused_neck)
+        e = launch_neck_max_head(nh, c->bf16, c->post);
+      else if (use_tc)
         e = launch_fuse_max_head(tp, c->bf16, c->post);
       else
         e = launch_fuse_head(fa, c->bf16, c->post);
@@ -963,7 +979,7 @@ rtcc_status capture_post(rtcc_ctx* c) {
   if (e == cudaSuccess && c->dec_boxes) e = launch_nms(na, c->post);
   if (e == cudaSuccess && tl) e = record_node(c->ev_post1, c->post);
   // fusion(s) and head, decode, NMS
-  c->post_kernels = (two_step ? (c->ms ? 3 : 2) : 1) + 1 + (c->dec_boxes ? 1 : 0);
+  c->post_kernels = (two_step ? (c->ms && !c->fused_neck ? 3 : 2) : 1) + 1 + (c->dec_boxes ? 1 : 0);
   cudaGraph_t graph = nullptr;
   cudaError_t e2 = cudaStreamEndCapture(c->post, &graph);
   if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -1783,6 +1799,19 @@ rtcc_status rtcc_get_pillars(rtcc_ctx* c, int32_t agent, int32_t* host_cell2pill
   return RTCC_OK;
 }
 
+// With the neck fused into the head's kernel no launch stores the feature
+// maps: run the deconvs of one agent (multi-scale: of the fused maps) over the
+// blocks' outputs of the last frame.  Mutex held, the branches' streams idle.
+static rtcc_status run_neck(rtcc_ctx* c, int agent) {
+  c->neck_p->agents[0] = c->ms ? 0 : agent;
+  CK(cudaStreamSynchronize(c->post));
+  CK(launch_backbone(*c->neck_p, c->bf16, c->bbst));
+  CK(cudaStreamSynchronize(c->bbst));
+  int err = 0;
+  CK(cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  return err ? RTCC_E_DEVICE : RTCC_OK;
+}
+
 rtcc_status rtcc_get_tensor(rtcc_ctx* c, int32_t agent, int32_t which, uint16_t* host_out,
                             size_t cap, size_t* n_elems) {
   if (!c) return RTCC_E_ARG;
@@ -1795,6 +1824,7 @@ rtcc_status rtcc_get_tensor(rtcc_ctx* c, int32_t agent, int32_t which, uint16_t*
     CK(cudaStreamSynchronize(c->post));
     src = f;
     n = (size_t)c->Wf * c->Hf * c->Cf;
+    if (host_out && cap >= n && c->fused_neck) RS(run_neck(c, 0));
   } else if (which >= 10 && which < 10 + c->cfg.n_blocks) {
     if (!c->ms) return RTCC_E_STATE;
     CK(cudaStreamSynchronize(c->post));
@@ -1815,6 +1845,7 @@ rtcc_status rtcc_get_tensor(rtcc_ctx* c, int32_t agent, int32_t which, uint16_t*
     } else if (which == 8) {
       src = b.feat;
       n = (size_t)c->Wf * c->Hf * c->Cf;
+      if (host_out && cap >= n && c->fused_neck && !c->ms) RS(run_neck(c, agent));
     } else if (which >= 16 && which - 16 < (int)c->layer_all.size() &&
                (c->cfg.flags & RTCC_FLAG_KEEP_LAYERS)) {
       n = c->layer_elems[which - 16];

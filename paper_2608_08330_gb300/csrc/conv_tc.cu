@@ -1043,43 +1043,42 @@ EncodeFn encode_fn() {
 
 }  // namespace
 
-cudaError_t tmap_2d(CUtensorMap* m, const void* base, bool bf16, uint64_t inner, uint64_t outer,
-                    uint32_t box_inner, uint32_t box_outer, int swizzle_bytes) {
+cudaError_t tmap_nd(CUtensorMap* m, const void* base, bool bf16, int rank, const uint64_t* dims,
+                    const uint64_t* strides, const uint32_t* box, int swizzle_bytes) {
   EncodeFn enc = encode_fn();
   if (!enc) return cudaErrorNotSupported;
+  if (rank < 2 || rank > 5) return cudaErrorInvalidValue;
   const CUtensorMapDataType dt =
       bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
   const CUtensorMapSwizzle sw = swizzle_bytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                                 : swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                       : CU_TENSOR_MAP_SWIZZLE_NONE;
-  cuuint64_t dims[2] = {inner, outer};
-  cuuint64_t strides[1] = {inner * 2};
-  cuuint32_t box[2] = {box_inner, box_outer};
-  cuuint32_t es[2] = {1, 1};
-  const CUresult r = enc(m, dt, 2, const_cast<void*>(base), dims, strides, box, es,
+  cuuint64_t d[5], s[4];
+  cuuint32_t b[5], es[5] = {1, 1, 1, 1, 1};
+  for (int i = 0; i < rank; ++i) {
+    d[i] = dims[i];
+    b[i] = box[i];
+    if (i + 1 < rank) s[i] = strides[i];
+  }
+  const CUresult r = enc(m, dt, (cuuint32_t)rank, const_cast<void*>(base), d, s, b, es,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t tmap_2d(CUtensorMap* m, const void* base, bool bf16, uint64_t inner, uint64_t outer,
+                    uint32_t box_inner, uint32_t box_outer, int swizzle_bytes) {
+  const uint64_t dims[2] = {inner, outer}, strides[1] = {inner * 2};
+  const uint32_t box[2] = {box_inner, box_outer};
+  return tmap_nd(m, base, bf16, 2, dims, strides, box, swizzle_bytes);
+}
+
 cudaError_t tmap_3d(CUtensorMap* m, const void* base, bool bf16, uint64_t inner, uint64_t mid,
                     uint64_t outer, uint32_t box_inner, uint32_t box_mid, uint32_t box_outer,
                     int swizzle_bytes) {
-  EncodeFn enc = encode_fn();
-  if (!enc) return cudaErrorNotSupported;
-  const CUtensorMapDataType dt =
-      bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  const CUtensorMapSwizzle sw = swizzle_bytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
-                                : swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                                      : CU_TENSOR_MAP_SWIZZLE_NONE;
-  cuuint64_t dims[3] = {inner, mid, outer};
-  cuuint64_t strides[2] = {inner * 2, inner * mid * 2};
-  cuuint32_t box[3] = {box_inner, box_mid, box_outer};
-  cuuint32_t es[3] = {1, 1, 1};
-  const CUresult r = enc(m, dt, 3, const_cast<void*>(base), dims, strides, box, es,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+  const uint64_t dims[3] = {inner, mid, outer}, strides[2] = {inner * 2, inner * mid * 2};
+  const uint32_t box[3] = {box_inner, box_mid, box_outer};
+  return tmap_nd(m, base, bf16, 3, dims, strides, box, swizzle_bytes);
 }
 
 int conv_tile_w() { return TW; }

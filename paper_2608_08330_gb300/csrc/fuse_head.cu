@@ -89,14 +89,6 @@ __device__ __forceinline__ void unpack(const uint32_t* r, float* x) {
   }
 }
 
-// ascending unsigned order of the result == descending float order; -0 -> +0
-__device__ __forceinline__ uint32_t ord_desc(float f) {
-  f = f + 0.0f;
-  const uint32_t u = __float_as_uint(f);
-  const uint32_t asc = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-  return ~asc;
-}
-
 // The fused vector of one cell for this lane's channels.
 template <typename T, int C, bool ATTN>
 __device__ __forceinline__ void fuse_cell(const T* const* slot, unsigned pres, int K, int cell,

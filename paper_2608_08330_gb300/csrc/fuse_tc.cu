@@ -67,24 +67,6 @@ __device__ __forceinline__ uint4 max8(uint4 a, uint4 b) {
   return make_uint4(max2<T>(a.x, b.x), max2<T>(a.y, b.y), max2<T>(a.z, b.z), max2<T>(a.w, b.w));
 }
 
-// ascending unsigned order of the result == descending float order; -0 -> +0
-__device__ __forceinline__ uint32_t ord_desc(float f) {
-  f = f + 0.0f;
-  const uint32_t u = __float_as_uint(f);
-  const uint32_t asc = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-  return ~asc;
-}
-
-// Count `key` (if `keep`) in the top-12-bit histogram: the lanes of a warp
-// that share a bin add their count with one atomic (valid logits crowd into
-// a few dozen bins, so per-key atomics would serialise on them).  Every lane
-// of the warp must call it.
-__device__ __forceinline__ void hist_add(uint32_t* hist0, bool keep, uint32_t key, int lane) {
-  const uint32_t bin = keep ? (key >> 20) : 0xFFFFFFFFu;
-  const unsigned peers = __match_any_sync(0xFFFFFFFFu, bin);
-  if (keep && lane == __ffs(peers) - 1) atomicAdd(&hist0[bin], (uint32_t)__popc(peers));
-}
-
 // Element-wise max of the KP present agents' copies of one staged chunk (nvec
 // 16-byte vectors each, agent i at st + i * nvec) into fb, by the worker
 // threads; 0 agents give zeros.  KP fixed at compile time lets the loads of

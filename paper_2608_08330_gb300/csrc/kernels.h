@@ -295,6 +295,62 @@ int fuse_tc_chunk(int C, int K);
 int fuse_tc_stages(int C, int K);   // pipeline stages for that chunk
 cudaError_t launch_fuse_max_head(const FuseTcParams& p, bool bf16, cudaStream_t st);
 
+// Neck (deconvs of every block), max over the agents and head in one kernel
+// (neck_head.cu), from the blocks' outputs.
+struct NeckHeadArgs {
+  int n_blocks;
+  const void* in[RTCC_MAX_BLOCKS];      // block b's outputs, agent-major [K][H_b][W_b][C_b]
+  long long astride[RTCC_MAX_BLOCKS];   // elements between agents
+  int cin[RTCC_MAX_BLOCKS];             // C_b
+  int stride[RTCC_MAX_BLOCKS];          // deconv kernel = stride
+  const void* w[RTCC_MAX_BLOCKS];       // packed deconv weights [s*s*128][C_b]
+  const float* bias[RTCC_MAX_BLOCKS];   // [128]
+  const void* head_w;                   // [16][128 n_blocks] in the storage type
+  int feat_w, feat_h;                   // output map
+  const int* present;                   // device [K]
+  int K;
+  const float* head_b;                  // device [16]
+  float* head_out;                      // device [cells][16]
+  uint32_t* keys;                       // device [cells][anchors] decode keys
+  uint32_t* hist0;                      // device [4096] top-12-bit key histogram
+  float cls_thresh;
+  int anchors;
+  int* err;
+  unsigned long long* span;             // device [3] kernel span stamps, or null
+  long long wait_budget;
+};
+struct NeckHeadParams {
+  CUtensorMap in[RTCC_MAX_BLOCKS];      // 5-D view (r C, W / r, r, H / r, agent), box (64, tw, 1, th, 1)
+  CUtensorMap w[RTCC_MAX_BLOCKS];       // deconv weights, box (64, 128)
+  CUtensorMap wh;                       // head weights, box (64, 16)
+  const float* bias[RTCC_MAX_BLOCKS];
+  int cin[RTCC_MAX_BLOCKS], s[RTCC_MAX_BLOCKS];
+  int n_blocks, S;                      // S: the largest deconv stride
+  int Wf, Wq, Hq;                       // output row length; quotient grid (W' / S, H' / S)
+  int tw, th, tiles_x, tiles;           // tiles of the quotient grid
+  int K;
+  const int* present;
+  const float* head_b;
+  float* head_out;
+  uint32_t* keys;
+  uint32_t* hist0;
+  float cls_thresh;
+  int anchors;
+  int* err;
+  unsigned long long* span;
+  long long wait_budget;
+};
+// Whether the kernel takes these blocks (64-channel chunks whose weights for
+// one position stay resident in shared memory).
+bool neck_head_ok(int n_blocks, const int* cin, const int* stride, int up_ch);
+void neck_head_tile(int W, int H, int* tw, int* th);
+cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P);
+cudaError_t launch_neck_max_head(const NeckHeadParams& p, bool bf16, cudaStream_t st);
+
+// Dense 16-bit tensor map of any rank up to 5 (dims innermost first, strides
+// in bytes of dimensions 1 .. rank - 1).
+cudaError_t tmap_nd(CUtensorMap* m, const void* base, bool bf16, int rank, const uint64_t* dims,
+                    const uint64_t* strides, const uint32_t* box, int swizzle_bytes);
 // Row-major 2-D 16-bit tensor map [outer][inner] with a box of
 // box_inner x box_outer elements and the given swizzle span (128, 64 or 0
 // bytes); OOB elements read as zero.

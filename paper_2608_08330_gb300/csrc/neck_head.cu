@@ -1,0 +1,527 @@
+// The deconv neck, the cross-agent max and the 1x1 detection head in one
+// kernel (the shared post-join subgraph, Sec. III-B / Sec. IV-D, for the
+// element-wise max fusion), on the 5th-generation tensor cores.
+//
+//   X_k[cell][128 b + c] = relu(bias_b[c] + sum_i W_b[sub][c][i] Y_kb[pixel][i])
+//   F[cell][.]           = max over present agents k of X_k[cell][.]
+//   out[cell][o]         = head_b[o] + sum_c W_head[o][c] F[cell][c],  o < 16
+//
+// with Y_kb agent k's output of backbone block b, pixel the input pixel under
+// the cell and sub the cell's position within it (kernel = stride = s_b).
+//
+// Why one kernel.  Run by the branches, the neck writes 384 channels per cell
+// and agent that the fusion then reads back: on the 352 x 100 map with 8
+// agents 2 x 216 MB through HBM, 125 us of deconvs behind the last conv (their
+// strided 128-channel stores bound them) and 48 us of fusion (0.67 of the
+// measured copy rate).  The blocks' outputs are 63 MB, mostly still in the
+// 129 MB L2, and the deconvs' 32 GFLOP are a fraction of the tensor cores'
+// time, so here the neck's output never leaves the SM.
+//
+// The maximum is taken on the fp32 accumulators, before bias, ReLU and the
+// rounding to 16 bits: all three are monotone, so rounding the maximum gives
+// the very bits of the maximum of the rounded values.
+//
+// Work item: 128 cells that share their position (sy, sx) modulo the largest
+// stride S, i.e. cells (S qy + sy, S qx + sx) of a tw x th rectangle of
+// (qx, qy).  They have one weight matrix per block -- 128 x C_b, all of them
+// resident in shared memory (112 KB for 64 + 128 + 256 channels) while the CTA
+// stays at that position -- and their pixels of block b form a dense
+// rectangle of a strided view of its map: one TMA box of 64 channels per
+// chunk (5-D view (r C, W / r, r, H / r, agent), r = S / s_b).  Items are
+// numbered position-major and each CTA takes a contiguous range.
+// The rectangle is the one that covers the map with the fewest tiles (88 x 25:
+// 5 x 25, 18 tiles against 22 of 8 x 16).
+//
+// Per item and block: for each present agent the block's chunks accumulate
+// into one of three 128-column accumulators; the epilogue keeps the running
+// maximum in registers (32 columns per thread); after the last agent it adds
+// the bias, applies ReLU, rounds and writes the 128 x 128 fused chunk as the A
+// operand of the head's N = 16 MMAs, which accumulate over the blocks in
+// channel order.
+//
+// Roles (800 threads): warps 0..15 max epilogue (tensor-memory lane quarter
+// warp % 4, columns 32 (warp / 4)), warps 16..19 head epilogue, warps 20..23
+// one TMA producer thread each (a thread's boxes complete one after another,
+// so the stages are dealt over four), warp 24 tensor-memory owner and MMA
+// issuer.  Every wait is bounded (an error bit, no hang); the summation order
+// is fixed, so the output is bit-reproducible.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace rtcc {
+
+namespace {
+
+constexpr int kEpiWarps = 16;
+constexpr int kHeadWarp0 = kEpiWarps;          // 4 head epilogue warps
+constexpr int kProdWarp0 = kHeadWarp0 + 4;
+constexpr int kProducers = 4;
+constexpr int kMmaWarp = kProdWarp0 + kProducers;
+constexpr int kThreads = (kMmaWarp + 1) * 32;
+constexpr int kStages = 4;                     // one per producer thread
+constexpr int kTile = 128;                     // cells per item (MMA M)
+constexpr int kUp = 128;                       // channels per deconv
+constexpr int kChunk = kTile * 64 * 2;         // 64 channels of 128 rows, 128-byte swizzle
+constexpr int kMaxChunks = 7;                  // weight chunks resident per position
+constexpr int kHeadChunk = kFuseHeadOut * 64 * 2;
+constexpr int kAccs = 3;
+constexpr uint32_t kHeadCol = kAccs * kUp;     // two 16-column head accumulators follow
+constexpr uint32_t kTmemCols = 512;
+// shared memory: A stages, resident weights, fused chunk pair, head weights
+constexpr int kWOff = kStages * kChunk;
+constexpr int kFOff = kWOff + kMaxChunks * kChunk;
+constexpr int kHOff = kFOff + 2 * kChunk;
+constexpr int kBarOff = kHOff + RTCC_MAX_BLOCKS * 2 * kHeadChunk;
+constexpr int kSmem = kBarOff + 256 + 1024;    // barriers; alignment to 1024
+static_assert(kSmem <= 227 * 1024 - 2048, "shared memory budget (with the static arrays)");
+static_assert(kStages == kProducers, "stage s belongs to producer thread s");
+
+// tile t of a CTA's range: position (sy, sx), origin in the quotient grid
+struct NhItem {
+  int sub, sy, sx, x0, y0;
+};
+__device__ __forceinline__ NhItem item_at(const NeckHeadParams& P, int t) {
+  NhItem I;
+  I.sub = t / P.tiles;
+  const int tau = t - I.sub * P.tiles;
+  I.sy = I.sub / P.S;
+  I.sx = I.sub - I.sy * P.S;
+  const int ty = tau / P.tiles_x;
+  I.x0 = (tau - ty * P.tiles_x) * P.tw;
+  I.y0 = ty * P.th;
+  return I;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_constant__ NeckHeadParams P) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint8_t* wsm = smem + kWOff;
+  uint8_t* fsm = smem + kFOff;
+  uint8_t* hsm = smem + kHOff;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kBarOff);   // [kStages]
+  uint64_t* empty = full + kStages;            // [kStages]
+  uint64_t* accfull = empty + kStages;         // [kAccs]
+  uint64_t* accempty = accfull + kAccs;        // [kAccs]
+  uint64_t* hfull = accempty + kAccs;          // [2] head accumulator complete
+  uint64_t* hempty = hfull + 2;                // [2]
+  uint64_t* wfull = hempty + 2;                // a position's weights landed
+  uint64_t* wempty = wfull + 1;                // the MMAs that read them are done
+  uint64_t* hwfull = wempty + 1;               // head weights landed
+  uint64_t* fready = hwfull + 1;               // fused chunk pair written
+  uint64_t* fempty = fready + 1;               // head MMAs have read it
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fempty + 1);
+  __shared__ __align__(16) float s_bias[RTCC_MAX_BLOCKS][kUp];
+  __shared__ int s_list[RTCC_MAX_AGENTS];
+  __shared__ int s_kp;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int nb = P.n_blocks;
+  const int n_items = P.S * P.S * P.tiles;
+  const int lo = (int)((long long)blockIdx.x * n_items / gridDim.x);
+  const int hi = (int)((long long)(blockIdx.x + 1) * n_items / gridDim.x);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int a = 0; a < kAccs; ++a) {
+      mbar_init(&accfull[a], 1);
+      mbar_init(&accempty[a], kEpiWarps);
+    }
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(&hfull[h], 1);
+      mbar_init(&hempty[h], 4);
+    }
+    mbar_init(wfull, kProducers);
+    mbar_init(wempty, 1);
+    mbar_init(hwfull, 1);
+    mbar_init(fready, kEpiWarps);
+    mbar_init(fempty, 1);
+    fence_barrier_init();
+  }
+  if (warp == kMmaWarp) {
+    tmem_alloc(tmem_slot, kTmemCols);
+    tmem_relinquish();
+  }
+  for (int i = threadIdx.x; i < nb * kUp; i += kThreads) s_bias[i / kUp][i % kUp] = P.bias[i / kUp][i % kUp];
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+
+  // Weights of position `sub`: producer thread pid issues every kProducers-th
+  // of the 64-channel chunks (blocks in order, chunk index running on).
+  auto load_weights = [&](const NhItem& I, int pid) {
+    uint32_t mine = 0;
+    int idx = 0;
+    for (int b = 0; b < nb; ++b)
+      for (int c = 0; c < P.cin[b] / 64; ++c, ++idx)
+        if (idx % kProducers == pid) mine += kChunk;
+    mbar_arrive_expect_tx(wfull, mine);
+    idx = 0;
+    for (int b = 0; b < nb; ++b) {
+      const int s = P.s[b];
+      const int row = ((I.sy % s) * s + I.sx % s) * kUp;
+      for (int c = 0; c < P.cin[b] / 64; ++c, ++idx)
+        if (idx % kProducers == pid) tma_load_2d(wsm + idx * kChunk, &P.w[b], wfull, c * 64, row);
+    }
+  };
+  // the weights are constant: the first position's loads overlap the previous kernel
+  const int pid = warp - kProdWarp0;
+  const bool producer = pid >= 0 && pid < kProducers && lane == 0;
+  if (producer && lo < hi) {
+    if (pid == 0) {
+      mbar_arrive_expect_tx(hwfull, (uint32_t)(nb * 2 * kHeadChunk));
+      for (int j = 0; j < nb * 2; ++j) tma_load_2d(hsm + j * kHeadChunk, &P.wh, hwfull, j * 64, 0);
+    }
+    load_weights(item_at(P, lo), pid);
+  }
+  pdl_wait();                                  // the maps are the branches' output
+  span_begin(P.span);
+  if (threadIdx.x == 0) {
+    int n = 0;
+    for (int k = 0; k < P.K; ++k)
+      if (P.present[k]) s_list[n++] = k;
+    s_kp = n;
+  }
+  __syncthreads();
+  const int Kp = s_kp;
+
+  if (warp < kEpiWarps) {
+    // ---------------- running max, bias + ReLU + rounding ----------------
+    const int qd = warp & 3, cg = warp >> 2;
+    const int row = qd * 32 + lane;
+    const uint32_t tcol = tmem + (static_cast<uint32_t>(qd * 32) << 16) + (uint32_t)(cg * 32);
+    // this thread's 32 channels of row `row` in the fused chunk pair: 16-byte
+    // pieces 4 (cg & 1) .. + 3 of the row in chunk cg / 2, 128-byte swizzle
+    uint8_t* frow = fsm + (cg >> 1) * kChunk + row * 128;
+    uint32_t st = 0, ph = 0;
+    bool alive = true;
+    for (int t = lo; t < hi; ++t) {
+      for (int b = 0; b < nb; ++b, ++ph) {
+        float mx[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) mx[i] = -INFINITY;
+        for (int k = 0; k < Kp; ++k, ++st) {
+          const uint32_t buf = st % kAccs;
+          if (alive && !mbar_wait(&accfull[buf], (st / kAccs) & 1, P.wait_budget)) {
+            if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
+            alive = false;
+          }
+          tc_fence_after();
+          uint32_t r0[16], r1[16];
+          tmem_ld16_issue(tcol + buf * kUp, r0);
+          tmem_ld16_issue(tcol + buf * kUp + 16, r1);
+          tmem_ld_wait();
+          tmem_reg_fence(r0);
+          tmem_reg_fence(r1);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&accempty[buf]);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            mx[i] = fmaxf(mx[i], __uint_as_float(r0[i]));
+            mx[16 + i] = fmaxf(mx[16 + i], __uint_as_float(r1[i]));
+          }
+        }
+        // the head MMAs of the previous block have read the fused chunk pair
+        if (alive && !mbar_wait(fempty, (ph & 1) ^ 1, P.wait_budget)) {
+          if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
+          alive = false;
+        }
+        const float4* bias = reinterpret_cast<const float4*>(&s_bias[b][cg * 32]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 ba = bias[2 * j], bb = bias[2 * j + 1];
+          const float* v = mx + 8 * j;
+          uint4 o;
+          o.x = Store<T>::pack2(relu_f(v[0] + ba.x), relu_f(v[1] + ba.y));
+          o.y = Store<T>::pack2(relu_f(v[2] + ba.z), relu_f(v[3] + ba.w));
+          o.z = Store<T>::pack2(relu_f(v[4] + bb.x), relu_f(v[5] + bb.y));
+          o.w = Store<T>::pack2(relu_f(v[6] + bb.z), relu_f(v[7] + bb.w));
+          *reinterpret_cast<uint4*>(frow + ((((cg & 1) * 4 + j) ^ (row & 7)) << 4)) = o;
+        }
+        fence_async_smem();                    // generic writes -> the MMA
+        __syncwarp();
+        if (lane == 0) mbar_arrive(fready);
+      }
+    }
+  } else if (warp < kProdWarp0) {
+    // ---------------- head epilogue ----------------
+    const int qd = warp & 3;
+    const int row = qd * 32 + lane;
+    const int ry = row / P.tw, rx = row - ry * P.tw;
+    float hb[kFuseHeadOut];
+#pragma unroll
+    for (int o = 0; o < kFuseHeadOut; ++o) hb[o] = P.head_b[o];
+    bool alive = true;
+    for (int t = lo; t < hi; ++t) {
+      const int n = t - lo, acc = n & 1;
+      const NhItem I = item_at(P, t);
+      if (alive && !mbar_wait(&hfull[acc], (n >> 1) & 1, P.wait_budget)) {
+        if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
+        alive = false;
+      }
+      tc_fence_after();
+      float v[16];
+      tmem_ld16(tmem + kHeadCol + acc * kFuseHeadOut + (static_cast<uint32_t>(qd * 32) << 16), v);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&hempty[acc]);
+      const int qx = I.x0 + rx, qy = I.y0 + ry;
+      const bool cv = ry < P.th && qx < P.Wq && qy < P.Hq;
+      const int cell = (qy * P.S + I.sy) * P.Wf + qx * P.S + I.sx;
+#pragma unroll
+      for (int o = 0; o < kFuseHeadOut; ++o) v[o] += hb[o];
+      if (cv) {
+        float4* ho = reinterpret_cast<float4*>(P.head_out + (size_t)cell * kFuseHeadOut);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ho[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      }
+#pragma unroll
+      for (int o = 0; o < kFuseHeadOut; ++o) {
+        if (o < P.anchors) {
+          const bool keep = cv && v[o] >= P.cls_thresh;
+          const uint32_t key = keep ? ord_desc(v[o]) : 0xFFFFFFFFu;
+          if (cv) P.keys[(size_t)cell * P.anchors + o] = key;
+          hist_add(P.hist0, keep, key, lane);
+        }
+      }
+    }
+  } else if (warp < kMmaWarp) {
+    // ---------------- TMA producers (one thread in each of 4 warps) ----------------
+    if (lane == 0 && lo < hi) {
+      const uint32_t bytes = (uint32_t)(P.tw * P.th * 128);
+      uint32_t it = 0, loads = 1, mine = 0;    // weight loads so far; A boxes of this thread
+      int cur = item_at(P, lo).sub;
+      bool alive = true;
+      for (int t = lo; t < hi && alive; ++t) {
+        const NhItem I = item_at(P, t);
+        if (I.sub != cur) {
+          // the MMAs that read the previous position's weights are done
+          if (!mbar_wait(wempty, (loads - 1) & 1, P.wait_budget)) {
+            alive = false;
+            break;
+          }
+          load_weights(I, pid);
+          ++loads;
+          cur = I.sub;
+        }
+        for (int b = 0; b < nb && alive; ++b) {
+          const int ox = I.sx / P.s[b], oy = I.sy / P.s[b];
+          const int nc = P.cin[b] / 64;
+          for (int k = 0; k < Kp && alive; ++k) {
+            const int agent = s_list[k];
+            for (int c = 0; c < nc; ++c, ++it) {
+              if ((int)(it % kProducers) != pid) continue;
+              if (!mbar_wait(&empty[pid], ((it / kStages) & 1) ^ 1, P.wait_budget)) {
+                alive = false;
+                break;
+              }
+              mbar_arrive_expect_tx(&full[pid], bytes);
+              tma_load_5d(smem + pid * kChunk, &P.in[b], &full[pid], ox * P.cin[b] + c * 64, I.x0, oy, I.y0,
+                          agent);
+              ++mine;
+            }
+          }
+        }
+      }
+      if (!alive) {
+        atomicOr(P.err, ERR_WAIT_FUSE);
+        // this thread's last box may still be in flight into the CTA's memory
+        if (mine > 0) (void)mbar_wait(&full[pid], (mine - 1) & 1, P.wait_budget);
+        (void)mbar_wait(wfull, (loads - 1) & 1, P.wait_budget);
+      }
+    }
+  } else if (lane == 0 && lo < hi) {
+    // ---------------- MMA issuer ----------------
+    const uint32_t idesc = idesc_f16(kTile, kUp, std::is_same<T, __nv_bfloat16>::value);
+    const uint32_t hdesc = idesc_f16(kTile, kFuseHeadOut, std::is_same<T, __nv_bfloat16>::value);
+    const uint32_t sm0 = smem_u32(smem);
+    uint32_t it = 0, st = 0, loads = 0, ph = 0;
+    int cur = -1;
+    bool alive = true;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      if (alive && !mbar_wait(bar, parity, P.wait_budget)) {
+        atomicOr(P.err, ERR_WAIT_FUSE);
+        alive = false;
+      }
+    };
+    wait(hwfull, 0);
+    // Head MMAs of a finished block (phase ph - 1): issued after the next
+    // step's MMAs, which keep the pipe busy while the epilogue writes the
+    // fused chunk.
+    bool pend = false;
+    int pb = 0, pn = 0;
+    uint32_t pph = 0;
+    auto flush = [&]() {
+      wait(fready, pph & 1);
+      if (pb == 0) wait(&hempty[pn & 1], ((pn >> 1) & 1) ^ 1);
+      if (!alive) return;
+      tc_fence_after();
+      const uint32_t d = tmem + kHeadCol + (pn & 1) * kFuseHeadOut;
+#pragma unroll
+      for (int kk = 0; kk < kUp / 16; ++kk) {
+        const uint64_t a = smem_desc(sm0 + kFOff + (kk / 4) * kChunk, 1024, 2) + 2 * (kk % 4);
+        const uint64_t w = smem_desc(sm0 + kHOff + (pb * 2 + kk / 4) * kHeadChunk, 1024, 2) + 2 * (kk % 4);
+        umma_f16(d, a, w, hdesc, (pb > 0 || kk > 0) ? 1u : 0u);
+      }
+      umma_commit(fempty);
+      if (pb == nb - 1) umma_commit(&hfull[pn & 1]);
+      pend = false;
+    };
+    for (int t = lo; t < hi && alive; ++t) {
+      const NhItem I = item_at(P, t);
+      if (I.sub != cur) {
+        if (cur >= 0) umma_commit(wempty);
+        wait(wfull, loads & 1);
+        ++loads;
+        cur = I.sub;
+      }
+      int w0 = 0;                              // block b's first weight chunk
+      for (int b = 0; b < nb && alive; ++b) {
+        const int nc = P.cin[b] / 64;
+        for (int k = 0; k < Kp && alive; ++k, ++st) {
+          const uint32_t buf = st % kAccs;
+          wait(&accempty[buf], ((st / kAccs) & 1) ^ 1);
+          tc_fence_after();
+          for (int c = 0; c < nc && alive; ++c, ++it) {
+            const uint32_t s = it % kStages;
+            wait(&full[s], (it / kStages) & 1);
+            if (!alive) break;
+            tc_fence_after();
+            const uint64_t a = smem_desc(sm0 + s * kChunk, 1024, 2);
+            const uint64_t w = smem_desc(sm0 + kWOff + (w0 + c) * kChunk, 1024, 2);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              umma_f16(tmem + buf * kUp, a + 2 * kk, w + 2 * kk, idesc, (c > 0 || kk > 0) ? 1u : 0u);
+            umma_commit(&empty[s]);
+          }
+          if (!alive) break;
+          umma_commit(&accfull[buf]);
+          if (pend) flush();
+        }
+        if (pend && alive) flush();            // no agent present
+        pend = true;
+        pb = b;
+        pn = t - lo;
+        pph = ph++;
+        w0 += nc;
+      }
+    }
+    if (pend && alive) flush();
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  span_end(P.span);
+  if (warp == kMmaWarp) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kTmemCols);
+  }
+}
+
+}  // namespace
+
+bool neck_head_ok(int n_blocks, const int* cin, const int* stride, int up_ch) {
+  if (n_blocks < 1 || n_blocks > RTCC_MAX_BLOCKS || up_ch != kUp) return false;
+  int chunks = 0, S = 1;
+  for (int b = 0; b < n_blocks; ++b) {
+    if (cin[b] < 64 || cin[b] % 64) return false;
+    if (stride[b] != 1 && stride[b] != 2 && stride[b] != 4) return false;
+    chunks += cin[b] / 64;
+    S = std::max(S, stride[b]);
+  }
+  return chunks <= kMaxChunks;
+}
+
+// The tw x th rectangle of at most 128 pixels that covers W x H with the
+// fewest tiles (the widest of those).
+void neck_head_tile(int W, int H, int* tw, int* th) {
+  long long best = -1;
+  for (int w = 1; w <= kTile && w <= W; ++w) {
+    const int h = std::min(kTile / w, H);
+    const long long n = (long long)((W + w - 1) / w) * ((H + h - 1) / h);
+    if (best < 0 || n <= best) {
+      best = n;
+      *tw = w;
+      *th = h;
+    }
+  }
+}
+
+cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P) {
+  if (!neck_head_ok(a.n_blocks, a.cin, a.stride, kUp) || a.K < 1 || a.K > RTCC_MAX_AGENTS ||
+      a.anchors < 1 || a.anchors > kFuseHeadOut || a.wait_budget < 1)
+    return cudaErrorInvalidValue;
+  std::memset(P, 0, sizeof(*P));
+  int S = 1;
+  for (int b = 0; b < a.n_blocks; ++b) S = std::max(S, a.stride[b]);
+  if (a.feat_w < S || a.feat_h < S || a.feat_w % S || a.feat_h % S) return cudaErrorInvalidValue;
+  P->n_blocks = a.n_blocks;
+  P->S = S;
+  P->Wf = a.feat_w;
+  P->Wq = a.feat_w / S;
+  P->Hq = a.feat_h / S;
+  neck_head_tile(P->Wq, P->Hq, &P->tw, &P->th);
+  P->tiles_x = (P->Wq + P->tw - 1) / P->tw;
+  P->tiles = P->tiles_x * ((P->Hq + P->th - 1) / P->th);
+  for (int b = 0; b < a.n_blocks; ++b) {
+    const int s = a.stride[b], r = S / s;
+    const uint64_t C = (uint64_t)a.cin[b], W = (uint64_t)(a.feat_w / s), H = (uint64_t)(a.feat_h / s);
+    if (a.astride[b] < (long long)(C * W * H) || (a.astride[b] * 2) % 16) return cudaErrorInvalidValue;
+    P->cin[b] = a.cin[b];
+    P->s[b] = s;
+    P->bias[b] = a.bias[b];
+    const uint64_t dims[5] = {(uint64_t)r * C, W / r, (uint64_t)r, H / r, (uint64_t)a.K};
+    const uint64_t strides[4] = {(uint64_t)r * C * 2, W * C * 2, (uint64_t)r * W * C * 2,
+                                 (uint64_t)a.astride[b] * 2};
+    const uint32_t box[5] = {64, (uint32_t)P->tw, 1, (uint32_t)P->th, 1};
+    cudaError_t e = tmap_nd(&P->in[b], a.in[b], bf16, 5, dims, strides, box, 128);
+    if (e != cudaSuccess) return e;
+    e = tmap_2d(&P->w[b], a.w[b], bf16, C, (uint64_t)(s * s * kUp), 64, kUp, 128);
+    if (e != cudaSuccess) return e;
+  }
+  const cudaError_t e =
+      tmap_2d(&P->wh, a.head_w, bf16, (uint64_t)(a.n_blocks * kUp), kFuseHeadOut, 64, kFuseHeadOut, 128);
+  if (e != cudaSuccess) return e;
+  P->K = a.K;
+  P->present = a.present;
+  P->head_b = a.head_b;
+  P->head_out = a.head_out;
+  P->keys = a.keys;
+  P->hist0 = a.hist0;
+  P->cls_thresh = a.cls_thresh;
+  P->anchors = a.anchors;
+  P->err = a.err;
+  P->span = a.span;
+  P->wait_budget = a.wait_budget;
+  return cudaSuccess;
+}
+
+cudaError_t launch_neck_max_head(const NeckHeadParams& p, bool bf16, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  // equal ranges: as many CTAs as keep the longest range at its minimum
+  const int items = p.S * p.S * p.tiles;
+  if (items < 1 || sms < 1) return cudaErrorInvalidValue;
+  const int rounds = (items + sms - 1) / sms;
+  const int grid = (items + rounds - 1) / rounds;
+  auto kern = bf16 ? k_neck_max_head<__nv_bfloat16> : k_neck_max_head<__half>;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3(grid), dim3(kThreads), kSmem, st, p);
+}
+
+}  // namespace rtcc

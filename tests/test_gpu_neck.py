@@ -1,0 +1,60 @@
+"""The post-join kernel that runs the deconv neck, the max over the agents and
+the head from the blocks' outputs, against the path that stores the neck's maps
+(RTCC_FLAG_KEEP_FUSED): the same sums, so the same bytes, for tiles that are
+ragged, single and narrow, one to three blocks, absent agents and both storage
+types; and the feature maps, which are then computed when they are read."""
+import dataclasses
+
+import pytest
+
+import synth
+from tests import gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    return U.load()
+
+
+def _cfg(w, h, agents, dtype="fp16", blocks=((1, 64, 2), (2, 128, 2), (1, 256, 2)), ups=(1, 2, 4), **kw):
+    hx, hy = 0.2 * w, 0.2 * h
+    base = synth.get_config("pp3")
+    return dataclasses.replace(
+        base, n_agents=agents, grid_w=w, grid_h=h, x_min=-hx, x_max=hx, y_min=-hy, y_max=hy,
+        pts_x=(-hx, hx), pts_y=(-hy, hy), n_uniform=3 * w, n_clusters=1, cluster_pts=50,
+        max_pillars=w * h, dtype=dtype, blocks=blocks, up_strides=ups, cls_thresh=-1.0, **kw)
+
+
+CASES = [
+    ("one tile of one pixel", _cfg(8, 8, 1), ()),
+    ("one wide row", _cfg(1040, 8, 2), ()),
+    ("one narrow column", _cfg(8, 1040, 2, "bf16"), ()),
+    ("ragged, several positions a CTA", _cfg(328, 184, 3, "bf16"), (1,)),
+    ("all agents, 25 rows", _cfg(704, 200, 8), ()),
+    ("all but one absent", _cfg(72, 40, 8), (0, 1, 2, 3, 4, 6, 7)),
+    ("one block", _cfg(40, 24, 3, blocks=((2, 128, 2),), ups=(1,)), ()),
+    ("two blocks, strides 2 and 4", _cfg(48, 40, 2, blocks=((1, 64, 1), (1, 256, 2)), ups=(1, 2)), ()),
+    ("multi-scale", _cfg(88, 56, 3, fusion="attn"), (2,)),
+]
+
+
+@pytest.mark.parametrize("cfg,absent", [c[1:] for c in CASES], ids=[c[0] for c in CASES])
+def test_neck_max_head_matches_the_stored_maps(R, cfg, absent):
+    scales = cfg.fusion == "attn"
+    flags = R.FLAG_MULTISCALE if scales else 0
+    pts = [synth.points_for(cfg, 0, k) for k in range(cfg.n_agents)]
+    got = []
+    for f in (flags, flags | R.FLAG_KEEP_FUSED):
+        ctx, _ = U.make_ctx(cfg, flags=f)
+        try:
+            for mode in (R.MODE_RTCC, R.MODE_BARRIER):
+                boxes = U.run_frame(ctx, cfg, pts, list(range(cfg.n_agents)), mode, absent=absent)
+                maps = ([R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED)] if scales else
+                        [R.rtcc_get_tensor(ctx, k, R.TENSOR_FEAT) for k in range(cfg.n_agents) if k not in absent])
+                got.append((R.rtcc_get_head(ctx, cfg.feat_h, cfg.feat_w).tobytes(), boxes.tobytes(),
+                            [m.tobytes() for m in maps]))
+        finally:
+            R.rtcc_destroy(ctx)
+    assert all(g == got[0] for g in got[1:])
