@@ -152,6 +152,28 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
   }
 }
 
+// The same for a whole warp in uniform control flow: every lane returns the
+// same answer, so the code after it stays warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, long long budget) {
+  if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+  const long long t0 = clock64();
+  while (true) {
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xFFFFFFFFu, clock64() - t0 > budget)) return false;
+  }
+}
+
+// One lane of a converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 // ---------------------------------------------------------------------------
 // TMA (tiled tensor copies global -> shared, completion on an mbarrier)
 // ---------------------------------------------------------------------------
@@ -360,6 +382,47 @@ __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+// One k-block of MMAs (BK = 64 or 32 -> 4 or 2 MMAs of K = 16).  The
+// issuing thread cannot issue an MMA before the tensor pipe takes the
+// previous one, so every instruction between them adds to the k-block's time;
+// one asm statement keeps that to one add per operand.  The descriptors come
+// as 32-bit halves: advancing K by 16 elements = 32 bytes is +2 in the
+// 16-byte address field of the low half (the start stays inside its stage,
+// so the field does not overflow), and the high half (stride, swizzle) is the
+// same for every MMA of an operand.
+__device__ __forceinline__ void mma_kblock(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                           uint32_t b_hi, uint32_t idesc, uint32_t acc0, bool bk64) {
+  if (bk64) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 al, bl;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "setp.eq.b32 q, %5, %5;\n\t"
+        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, p;\n\t"
+        "add.u32 al, %1, 2;\n\tadd.u32 bl, %3, 2;\n\t"
+        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t"
+        "add.u32 al, %1, 4;\n\tadd.u32 bl, %3, 4;\n\t"
+        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t"
+        "add.u32 al, %1, 6;\n\tadd.u32 bl, %3, 6;\n\t"
+        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(acc0), "r"(idesc));
+  } else {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 al, bl;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "setp.eq.b32 q, %5, %5;\n\t"
+        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, p;\n\t"
+        "add.u32 al, %1, 2;\n\tadd.u32 bl, %3, 2;\n\t"
+        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(acc0), "r"(idesc));
+  }
 }
 
 // Arrive once on `bar` when every tcgen05 op this thread issued so far is done.

@@ -331,47 +331,6 @@ __device__ __forceinline__ void load_halo(const CUtensorMap* map, uint8_t* dH, u
   tma_load_4d(dH, map, bar, cb * 64, I.x0 - 1, I.y0 - 1, I.agent);
 }
 
-// One k-block of MMAs (BK = 64 or 32 -> 4 or 2 MMAs of K = 16).  The
-// issuing thread cannot issue an MMA before the tensor pipe takes the
-// previous one, so every instruction between them adds to the k-block's time;
-// one asm statement keeps that to one add per operand.  The descriptors come
-// as 32-bit halves: advancing K by 16 elements = 32 bytes is +2 in the
-// 16-byte address field of the low half (the start stays inside its stage,
-// so the field does not overflow), and the high half (stride, swizzle) is the
-// same for every MMA of an operand.
-__device__ __forceinline__ void mma_kblock(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                           uint32_t b_hi, uint32_t idesc, uint32_t acc0, bool bk64) {
-  if (bk64) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 al, bl;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "setp.eq.b32 q, %5, %5;\n\t"
-        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, p;\n\t"
-        "add.u32 al, %1, 2;\n\tadd.u32 bl, %3, 2;\n\t"
-        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t"
-        "add.u32 al, %1, 4;\n\tadd.u32 bl, %3, 4;\n\t"
-        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t"
-        "add.u32 al, %1, 6;\n\tadd.u32 bl, %3, 6;\n\t"
-        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t}" ::"r"(d_tmem),
-        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(acc0), "r"(idesc));
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t.reg .b32 al, bl;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "setp.eq.b32 q, %5, %5;\n\t"
-        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, p;\n\t"
-        "add.u32 al, %1, 2;\n\tadd.u32 bl, %3, 2;\n\t"
-        "mov.b64 a, {al, %2};\n\tmov.b64 b, {bl, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %6, q;\n\t}" ::"r"(d_tmem),
-        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(acc0), "r"(idesc));
-  }
-}
-
 // The MMAs of one 64-channel chunk of a halo layer's item: the 9 taps fully
 // unrolled, so every descriptor offset is an immediate and the MMAs issue
 // back to back; a stage of kpb taps (km = kpb - 1) starts with a wait on its
@@ -379,20 +338,21 @@ __device__ __forceinline__ void mma_kblock(uint32_t d_tmem, uint32_t a_lo, uint3
 // row block (accumulator columns +128) takes the same weight box with the A
 // rows TH halo rows further down.  TR: the halo tile is stored in transposed
 // tile coordinates (tile x along the image's H), so image tap (dy, dx) starts
-// dx * kHaloW + dy rows into it instead of dy * kHaloW + dx.  False if a wait
-// runs out.
+// dx * kHaloW + dy rows into it instead of dy * kHaloW + dx.  Run by the whole
+// MMA warp in uniform control flow, one elected lane (leader) issuing.  False
+// if a wait runs out.
 template <bool TALL, bool TR>
 __device__ __forceinline__ bool halo_chunk_mma(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo0,
                                                uint32_t b_hi, uint32_t idesc, int km, uint32_t bstep,
                                                bool accumulate, uint64_t* full, uint64_t* empty, uint32_t& it,
-                                               long long budget) {
+                                               bool leader, long long budget) {
   uint32_t b_lo = 0;
   int s = 0;
 #pragma unroll
   for (int tap = 0; tap < 9; ++tap) {
     if ((tap & km) == 0) {
       s = it % kStages;
-      if (!mbar_wait(&full[s], (it / kStages) & 1, budget)) return false;
+      if (!mbar_wait_warp(&full[s], (it / kStages) & 1, budget)) return false;
       tc_fence_after();
       b_lo = b_lo0 + (uint32_t)(s * (kBBytes >> 4));
     }
@@ -400,12 +360,14 @@ __device__ __forceinline__ bool halo_chunk_mma(uint32_t d_tmem, uint32_t a_lo, u
     const uint32_t a_tap = a_lo + (uint32_t)((tap_y * kHaloW + tap_x) * 8);
     const uint32_t b_tap = b_lo + (uint32_t)(tap & km) * bstep;
     const uint32_t accum = (accumulate || tap > 0) ? 1u : 0u;
-    mma_kblock(d_tmem, a_tap, a_hi, b_tap, b_hi, idesc, accum, true);
-    if (TALL) mma_kblock(d_tmem + 128, a_tap + kTallHalfDesc, a_hi, b_tap, b_hi, idesc, accum, true);
-    if (((tap + 1) & km) == 0 || tap == 8) {
-      umma_commit(&empty[s]);
-      ++it;
+    const bool ends = ((tap + 1) & km) == 0 || tap == 8;
+    if (leader) {
+      mma_kblock(d_tmem, a_tap, a_hi, b_tap, b_hi, idesc, accum, true);
+      if (TALL) mma_kblock(d_tmem + 128, a_tap + kTallHalfDesc, a_hi, b_tap, b_hi, idesc, accum, true);
+      if (ends) umma_commit(&empty[s]);
     }
+    __syncwarp();
+    if (ends) ++it;
   }
   return true;
 }
@@ -429,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
   __shared__ int s_agents[RTCC_MAX_AGENTS];    // the launch's agents (batch slot -> agent)
   const long long budget = P.wait_budget;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
   const int lane = threadIdx.x & 31;
   // The DSMEM reduction needs the launch to be in clusters of kMaxSplits CTAs;
   // the cluster size is read from the hardware, not trusted from the
@@ -641,87 +603,98 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer (one thread) ----------------
-      uint32_t it = 0, tc = 0, hc = 0;
-      bool alive = true;
-      const uint32_t smem0 = smem_u32(smem);
-      for (int l = 0; l < P.n_layers && alive; ++l) {
-        const LayerScalars S = layer_scalars(P.L[l], P.n_batch);
-        const uint32_t idesc = idesc_f16(BM, S.bn, std::is_same<T, __nv_bfloat16>::value);
-        const bool bk64 = S.bk == 64;
-        const uint32_t swz = bk64 ? 2u : 4u;            // 128B : 64B swizzle
-        const uint32_t sbo = 8u * S.bk * 2u;            // bytes between 8-row atoms
-        // descriptor halves of the first A and B slots (the slots of a stage
-        // s are kABytes / kBBytes further on) and of the halo slots
-        const uint64_t ad0 = smem_desc(smem0, sbo, swz), bd0 = smem_desc(smem0 + kBOff, sbo, swz);
-        const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32);
-        const uint32_t b_lo0 = (uint32_t)bd0, b_hi = (uint32_t)(bd0 >> 32);
-        const uint32_t a_hi_halo = (uint32_t)(smem_desc(smem0, kHaloW * 128, 2u) >> 32);
-        const int t0 = first_item(S), tstep = S.cta_hi - S.cta_lo;
-        for (int t = t0; t >= 0 && t < S.n_items && alive; t += tstep, ++tc) {
-          const Item I = item_of(S, t, s_agents);
-          const int acc = tc & 1;
-          if (!mbar_wait(&accempty[acc], ((tc >> 1) & 1) ^ 1, budget)) {
-            atomicOr(P.err, ERR_WAIT_MMA);
-            alive = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d_tmem = tmem + acc * kAccStride;
-          if (S.halo) {
-            // Chunk by chunk: wait for the halo tile, then the 9 taps fully
-            // unrolled, so every descriptor offset is an immediate and the
-            // MMAs issue back to back; a stage of kpb taps starts with a wait
-            // on its weight boxes and ends with a commit that frees it.  A
-            // tall tile's lower row block (accumulator columns +128) takes the
-            // same weight box with the A rows TH halo rows further down.
-            const bool tall = S.tall != 0;
-            const int nch = (I.kb1 - I.kb0) / 9;
-            const int km = S.kpb - 1;
-            const uint32_t bstep = (uint32_t)(S.bn * 8);        // one weight box, 16-byte units
-            for (int c = 0; c < nch && alive; ++c) {
-              const int h = hc % kHalo;
-              if (!mbar_wait(&hfull[h], (hc / kHalo) & 1, budget)) {
-                atomicOr(P.err, ERR_WAIT_MMA);
-                alive = false;
-                break;
-              }
-              ++hc;
-              const uint32_t a_lo = (uint32_t)smem_desc(smem0 + h * kHaloSlot, kHaloW * 128, 2u);
-              const bool acc_in = c > 0;
-              const bool ok =
-                  tall ? (S.tr ? halo_chunk_mma<true, true>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km, bstep,
-                                                            acc_in, full, empty, it, budget)
-                               : halo_chunk_mma<true, false>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
-                                                             bstep, acc_in, full, empty, it, budget))
-                       : (S.tr ? halo_chunk_mma<false, true>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
-                                                             bstep, acc_in, full, empty, it, budget)
-                               : halo_chunk_mma<false, false>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
-                                                              bstep, acc_in, full, empty, it, budget));
-              if (!ok) {
-                atomicOr(P.err, ERR_WAIT_MMA);
-                alive = false;
-                break;
-              }
-              umma_commit(&hempty[h]);
+    // ---------------- MMA issuer (the whole warp, one elected lane issuing) ----------------
+    // The MMA takes its descriptors from uniform registers.  Issued from a
+    // branch that one lane takes, an MMA cost 110 to 150 clocks of issue, more
+    // than its 45 to 64 in the pipe; with the warp converged (waits end with a
+    // vote, only the issue is predicated) an N = 128 MMA takes 64 to 75.  On
+    // the 704 x 200 grid the one-agent launch went from 133 to 116 us, the
+    // 8-agent one from 407 to 370 us.  (Testing the next stage's barrier ahead
+    // of the MMAs, or the whole ring's with one ballot, gained nothing here.)
+    const bool leader = elect_one();
+    uint32_t it = 0, tc = 0, hc = 0;
+    bool alive = true;
+    const uint32_t smem0 = smem_u32(smem);
+    for (int l = 0; l < P.n_layers && alive; ++l) {
+      const LayerScalars S = layer_scalars(P.L[l], P.n_batch);
+      const uint32_t idesc = idesc_f16(BM, S.bn, std::is_same<T, __nv_bfloat16>::value);
+      const bool bk64 = S.bk == 64;
+      const uint32_t swz = bk64 ? 2u : 4u;            // 128B : 64B swizzle
+      const uint32_t sbo = 8u * S.bk * 2u;            // bytes between 8-row atoms
+      // descriptor halves of the first A and B slots (the slots of a stage
+      // s are kABytes / kBBytes further on) and of the halo slots
+      const uint64_t ad0 = smem_desc(smem0, sbo, swz), bd0 = smem_desc(smem0 + kBOff, sbo, swz);
+      const uint32_t a_lo0 = (uint32_t)ad0, a_hi = (uint32_t)(ad0 >> 32);
+      const uint32_t b_lo0 = (uint32_t)bd0, b_hi = (uint32_t)(bd0 >> 32);
+      const uint32_t a_hi_halo = (uint32_t)(smem_desc(smem0, kHaloW * 128, 2u) >> 32);
+      const int t0 = first_item(S), tstep = S.cta_hi - S.cta_lo;
+      for (int t = t0; t >= 0 && t < S.n_items && alive; t += tstep, ++tc) {
+        const Item I = item_of(S, t, s_agents);
+        const int acc = tc & 1;
+        if (!mbar_wait_warp(&accempty[acc], ((tc >> 1) & 1) ^ 1, budget)) {
+          if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
+          alive = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d_tmem = tmem + acc * kAccStride;
+        if (S.halo) {
+          // Chunk by chunk: wait for the halo tile, then the 9 taps fully
+          // unrolled, so every descriptor offset is an immediate and the
+          // MMAs issue back to back; a stage of kpb taps starts with a wait
+          // on its weight boxes and ends with a commit that frees it.  A
+          // tall tile's lower row block (accumulator columns +128) takes the
+          // same weight box with the A rows TH halo rows further down.
+          const bool tall = S.tall != 0;
+          const int nch = (I.kb1 - I.kb0) / 9;
+          const int km = S.kpb - 1;
+          const uint32_t bstep = (uint32_t)(S.bn * 8);        // one weight box, 16-byte units
+          for (int c = 0; c < nch && alive; ++c) {
+            const int h = hc % kHalo;
+            if (!mbar_wait_warp(&hfull[h], (hc / kHalo) & 1, budget)) {
+              if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
+              alive = false;
+              break;
             }
-          } else {
-            for (int kb = I.kb0; kb < I.kb1; ++kb, ++it) {
-              const int s = it % kStages;
-              if (!mbar_wait(&full[s], (it / kStages) & 1, budget)) {
-                atomicOr(P.err, ERR_WAIT_MMA);
-                alive = false;
-                break;
-              }
-              tc_fence_after();
+            ++hc;
+            const uint32_t a_lo = (uint32_t)smem_desc(smem0 + h * kHaloSlot, kHaloW * 128, 2u);
+            const bool acc_in = c > 0;
+            const bool ok =
+                tall ? (S.tr ? halo_chunk_mma<true, true>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km, bstep,
+                                                          acc_in, full, empty, it, leader, budget)
+                             : halo_chunk_mma<true, false>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
+                                                           bstep, acc_in, full, empty, it, leader, budget))
+                     : (S.tr ? halo_chunk_mma<false, true>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
+                                                           bstep, acc_in, full, empty, it, leader, budget)
+                             : halo_chunk_mma<false, false>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
+                                                            bstep, acc_in, full, empty, it, leader, budget));
+            if (!ok) {
+              if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
+              alive = false;
+              break;
+            }
+            if (leader) umma_commit(&hempty[h]);
+            __syncwarp();
+          }
+        } else {
+          for (int kb = I.kb0; kb < I.kb1; ++kb, ++it) {
+            const int s = it % kStages;
+            if (!mbar_wait_warp(&full[s], (it / kStages) & 1, budget)) {
+              if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
+              alive = false;
+              break;
+            }
+            tc_fence_after();
+            if (leader) {
               mma_kblock(d_tmem, a_lo0 + (uint32_t)(s * (kABytes >> 4)), a_hi,
                          b_lo0 + (uint32_t)(s * (kBBytes >> 4)), b_hi, idesc, kb > I.kb0 ? 1u : 0u, bk64);
               umma_commit(&empty[s]);
             }
+            __syncwarp();
           }
-          umma_commit(&accfull[acc]);
         }
+        if (leader) umma_commit(&accfull[acc]);
+        __syncwarp();
       }
     }
   } else {

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
   __shared__ int s_list[RTCC_MAX_AGENTS];
   __shared__ int s_kp;
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
   const int lane = threadIdx.x & 31;
   const int nb = P.n_blocks;
   const int n_items = P.S * P.S * P.tiles;
@@ -342,83 +342,87 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
         (void)mbar_wait(wfull, (loads - 1) & 1, P.wait_budget);
       }
     }
-  } else if (lane == 0 && lo < hi) {
-    // ---------------- MMA issuer ----------------
+  } else if (lo < hi) {
+    // ---------------- MMA issuer (the whole warp, one elected lane issuing) ----------------
+    // The MMA's descriptors have to be in uniform registers: issued from a
+    // branch that one lane takes, each of a chunk's 4 MMAs cost about 150
+    // clocks (64 in the pipe).  So the warp stays converged -- waits end with
+    // a vote -- and only the issue itself is predicated: 8 agents on the
+    // 352 x 100 map 53.6 -> 40.9 us.
     const uint32_t idesc = idesc_f16(kTile, kUp, std::is_same<T, __nv_bfloat16>::value);
     const uint32_t hdesc = idesc_f16(kTile, kFuseHeadOut, std::is_same<T, __nv_bfloat16>::value);
-    const uint32_t sm0 = smem_u32(smem);
+    const uint64_t d0 = smem_desc(smem_u32(smem), 1024, 2);
+    const uint32_t lo0 = (uint32_t)d0, hi0 = (uint32_t)(d0 >> 32);   // operands differ in the address only
+    const long long budget = P.wait_budget;
+    const bool leader = elect_one();
     uint32_t it = 0, st = 0, loads = 0, ph = 0;
     int cur = -1;
-    bool alive = true;
-    auto wait = [&](uint64_t* bar, uint32_t parity) {
-      if (alive && !mbar_wait(bar, parity, P.wait_budget)) {
-        atomicOr(P.err, ERR_WAIT_FUSE);
-        alive = false;
-      }
-    };
-    wait(hwfull, 0);
-    // Head MMAs of a finished block (phase ph - 1): issued after the next
-    // step's MMAs, which keep the pipe busy while the epilogue writes the
-    // fused chunk.
+    bool alive = mbar_wait_warp(hwfull, 0, budget);
+    // Head MMAs of a finished block (phase pph): issued after the next step's
+    // MMAs, which keep the pipe busy while the epilogue writes the fused chunk.
     bool pend = false;
     int pb = 0, pn = 0;
     uint32_t pph = 0;
     auto flush = [&]() {
-      wait(fready, pph & 1);
-      if (pb == 0) wait(&hempty[pn & 1], ((pn >> 1) & 1) ^ 1);
-      if (!alive) return;
+      pend = false;
+      if (!mbar_wait_warp(fready, pph & 1, budget) ||
+          (pb == 0 && !mbar_wait_warp(&hempty[pn & 1], ((pn >> 1) & 1) ^ 1, budget))) {
+        alive = false;
+        return;
+      }
       tc_fence_after();
       const uint32_t d = tmem + kHeadCol + (pn & 1) * kFuseHeadOut;
+      if (leader) {
 #pragma unroll
-      for (int kk = 0; kk < kUp / 16; ++kk) {
-        const uint64_t a = smem_desc(sm0 + kFOff + (kk / 4) * kChunk, 1024, 2) + 2 * (kk % 4);
-        const uint64_t w = smem_desc(sm0 + kHOff + (pb * 2 + kk / 4) * kHeadChunk, 1024, 2) + 2 * (kk % 4);
-        umma_f16(d, a, w, hdesc, (pb > 0 || kk > 0) ? 1u : 0u);
+        for (int q = 0; q < 2; ++q)
+          mma_kblock(d, lo0 + ((kFOff + q * kChunk) >> 4), hi0,
+                     lo0 + ((kHOff + (pb * 2 + q) * kHeadChunk) >> 4), hi0, hdesc, (pb > 0 || q > 0) ? 1u : 0u,
+                     true);
+        umma_commit(fempty);
+        if (pb == nb - 1) umma_commit(&hfull[pn & 1]);
       }
-      umma_commit(fempty);
-      if (pb == nb - 1) umma_commit(&hfull[pn & 1]);
-      pend = false;
+      __syncwarp();
     };
     for (int t = lo; t < hi && alive; ++t) {
-      const NhItem I = item_at(P, t);
-      if (I.sub != cur) {
-        if (cur >= 0) umma_commit(wempty);
-        wait(wfull, loads & 1);
+      const int sub = t / P.tiles;
+      if (sub != cur) {
+        if (cur >= 0 && leader) umma_commit(wempty);
+        alive = mbar_wait_warp(wfull, loads & 1, budget);
         ++loads;
-        cur = I.sub;
+        cur = sub;
       }
-      int w0 = 0;                              // block b's first weight chunk
+      uint32_t w_lo = lo0 + (kWOff >> 4);      // block b's first weight chunk
       for (int b = 0; b < nb && alive; ++b) {
         const int nc = P.cin[b] / 64;
         for (int k = 0; k < Kp && alive; ++k, ++st) {
           const uint32_t buf = st % kAccs;
-          wait(&accempty[buf], ((st / kAccs) & 1) ^ 1);
-          tc_fence_after();
+          alive = mbar_wait_warp(&accempty[buf], ((st / kAccs) & 1) ^ 1, budget);
+          const uint32_t d = tmem + buf * kUp;
           for (int c = 0; c < nc && alive; ++c, ++it) {
             const uint32_t s = it % kStages;
-            wait(&full[s], (it / kStages) & 1);
+            alive = mbar_wait_warp(&full[s], (it / kStages) & 1, budget);
             if (!alive) break;
             tc_fence_after();
-            const uint64_t a = smem_desc(sm0 + s * kChunk, 1024, 2);
-            const uint64_t w = smem_desc(sm0 + kWOff + (w0 + c) * kChunk, 1024, 2);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_f16(tmem + buf * kUp, a + 2 * kk, w + 2 * kk, idesc, (c > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(&empty[s]);
+            if (leader) {
+              mma_kblock(d, lo0 + s * (kChunk >> 4), hi0, w_lo + c * (kChunk >> 4), hi0, idesc, c > 0 ? 1u : 0u,
+                         true);
+              umma_commit(&empty[s]);
+              if (c == nc - 1) umma_commit(&accfull[buf]);
+            }
+            __syncwarp();
           }
-          if (!alive) break;
-          umma_commit(&accfull[buf]);
-          if (pend) flush();
+          if (pend && alive) flush();
         }
         if (pend && alive) flush();            // no agent present
         pend = true;
         pb = b;
         pn = t - lo;
         pph = ph++;
-        w0 += nc;
+        w_lo += nc * (kChunk >> 4);
       }
     }
     if (pend && alive) flush();
+    if (!alive && lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
   }
 
   tc_fence_before();
