@@ -92,11 +92,14 @@ typedef enum {
                                     so each can be read back (parity)         */
 #define RTCC_FLAG_LAYER_TIMES 8  /* record the GPU times at which the backbone
                                     kernel starts and ends each conv/deconv
-                                    layer                                     */
+                                    layer (a layer then waits for all agents
+                                    of the launch, and the branches run the
+                                    neck themselves)                          */
 #define RTCC_FLAG_NO_CLUSTERS 16 /* launch the backbone without thread-block
-                                    clusters: split-K slices then reduce
-                                    through global memory instead of
-                                    distributed shared memory (same results)  */
+                                    clusters: one CTA then takes all split-K
+                                    slices of a tile instead of four that
+                                    exchange them through distributed shared
+                                    memory (same results)                     */
 #define RTCC_FLAG_SHORT_WAITS 32 /* bounded device waits give up after about
                                     10 ms instead of about 1 s, and
                                     rtcc_test_unreachable_wait is enabled
@@ -503,8 +506,11 @@ typedef struct {
 } rtcc_conv_plan;
 
 /*
- * The tile choice rtcc_init makes for one 3x3 conv layer (pad 1) of a
- * backbone launch over n_batch agents on `grid` CTAs: kind 0 = stride 1,
+ * The tile choice for one 3x3 conv layer (pad 1) of a backbone launch over
+ * n_batch agents on `grid` CTAs whose layers wait for each other, as rtcc_init
+ * makes it for n_batch = 1 (launches over several agents flow from layer to
+ * layer; rtcc_init then counts items / grid, at least 1, in place of whole
+ * rounds): kind 0 = stride 1,
  * 1 = stride 2; cin, cout its channels; out_w x out_h its output.  The K
  * slices come from the one-agent cost model, the N tile and tile shape from
  * the cost model at n_batch (rounds of items over the grid x k-blocks per

@@ -44,8 +44,6 @@ struct Branch {
   PillarBufs pb{};
   void* feat = nullptr;            // agent-indexed feature slot [H'][W'][C_feat] (a view
                                    // into the context's feature slots)
-  float* splitk_ws = nullptr;      // split-K partials of this branch's own launches
-  int* splitk_cnt = nullptr;       // split-K per-tile arrival counters
   unsigned* grid_bar = nullptr;      // inside frame_zero: per-layer counters + exit count
   void* frame_zero = nullptr;         // [kFrameZeroBytes] cleared by every pass's first pillar kernel
   unsigned long long* stamps = nullptr;   // RTCC_FLAG_LAYER_TIMES: layer starts, then ends
@@ -106,7 +104,7 @@ struct rtcc_ctx {
   void* neck_out = nullptr;           // neck of the fused blocks [H'][W'][C_feat]
   std::vector<ConvLayer> neck_layers; // the deconvs, when they are not layers of the branches
   BackboneParams* neck_p = nullptr;
-  unsigned* neck_bar = nullptr;       // [kMaxLayers + 1], zero between launches
+  unsigned* neck_bar = nullptr;       // [kBarWords], zero between launches
   int* d_one = nullptr;               // [RTCC_MAX_AGENTS] = {1, 0, ...}: the head's one input
   int post_kernels = 0;               // kernels of the post-join graph
   size_t img_elems = 0, feat_elems = 0;
@@ -115,9 +113,7 @@ struct rtcc_ctx {
   long long wait_budget = 0;
   // batched backbone launches (agents released together)
   cudaStream_t bbst = nullptr;
-  float* batch_ws = nullptr;
-  int* batch_cnt = nullptr;
-  unsigned* batch_bar = nullptr;      // [kMaxLayers + 1], zero between launches
+  unsigned* batch_bar = nullptr;      // [kBarWords], zero between launches
   cudaEvent_t batch_ev[RTCC_MAX_AGENTS] = {}, batch_t0[RTCC_MAX_AGENTS] = {},
               batch_t1[RTCC_MAX_AGENTS] = {};
   BackboneParams* launch_p = nullptr; // scratch for one launch's parameters
@@ -136,7 +132,6 @@ struct rtcc_ctx {
   int dev = 0;
   volatile int* stall = nullptr;      // pinned test hook word (RTCC_FLAG_SHORT_WAITS)
   bool disp_err = false;              // the dispatcher failed to launch a batch
-  size_t splitk_cnt_bytes = 0;        // split-K tile counters of one branch (batch: K x)
   cudaStream_t xfer = nullptr, post = nullptr;
   cudaGraphExec_t post_exec = nullptr;
   int* d_present = nullptr;           // [K] set by a branch's first kernel, cleared by the decode
@@ -397,7 +392,7 @@ void pick_tile(int m_tiles, int co, int total_kb, int grid, int* bn_out, int* sp
   *sp_out = bs;
 }
 
-constexpr size_t kFrameZeroBytes = 8 * sizeof(int) + (kMaxLayers + 1) * sizeof(unsigned);
+constexpr size_t kFrameZeroBytes = 8 * sizeof(int) + kBarWords * sizeof(unsigned);
 
 // Tile of a conv layer in a launch over `batch` agents, with its K slices
 // fixed (they decide the fp32 summation order, so they are the same for every
@@ -418,7 +413,13 @@ constexpr size_t kFrameZeroBytes = 8 * sizeof(int) + (kMaxLayers + 1) * sizeof(u
 // first orientation.
 constexpr double kTallCost = 1.6;
 double kblock_cost(int bn) { return bn >= 128 ? 1.0 : bn >= 64 ? 0.75 : 0.70; }
-void pick_tile_batch(const ConvLayer L0, int sp, int grid, int batch, bool need64, ConvLayer* out) {
+//
+// `flow`: rounds are counted as items / grid, at least 1, instead of whole
+// rounds.  In a launch over several agents the layers' items follow each other
+// round-robin without a barrier between layers, so a layer's last, partly
+// filled round costs its share only; a layer with fewer items than CTAs still
+// takes an item's time.
+void pick_tile_batch(const ConvLayer L0, int sp, int grid, int batch, bool need64, bool flow, ConvLayer* out) {
   double best = 1e30;
   out->bn = std::min(L0.cout, 64);
   out->tall = out->tr = out->wide = 0;
@@ -436,7 +437,7 @@ void pick_tile_batch(const ConvLayer L0, int sp, int grid, int batch, bool need6
         L.wide = orient && !halo;
         if (!conv_shape_ok(L)) continue;
         const int items = batch * conv_m_tiles(L) * (L.cout / bn) * sp;
-        const int rounds = (items + grid - 1) / grid;
+        const double rounds = flow ? std::max(1.0, (double)items / grid) : (double)((items + grid - 1) / grid);
         const double cost =
             rounds * (double)((total_kb + sp - 1) / sp) * kblock_cost(bn) * (tall ? kTallCost : 1.0);
         if (cost < best - 1e-9) {
@@ -462,13 +463,22 @@ void choose_split(ConvLayer& L, int grid) {
 }
 
 // The N tile and tile shape of conv layer L (K slices already chosen) in a
-// launch over nb agents.  A split layer whose items fit the clustered grid
-// keeps the DSMEM exchange (64-wide tiles); otherwise it reduces through
-// global memory.
+// launch over nb agents whose layers wait for each other.  A split layer whose
+// items fit the clustered grid keeps 64-wide tiles, which the DSMEM exchange
+// takes.
 void choose_tiles(ConvLayer& L, int grid, int nb) {
   const int m_tiles = conv_m_tiles(L);
   const bool dsm_fit = L.splits > 1 && nb * m_tiles * (L.cout / 64) * L.splits <= grid;
-  pick_tile_batch(L, L.splits, grid, nb, dsm_fit, &L);
+  pick_tile_batch(L, L.splits, grid, nb, dsm_fit, false, &L);
+  L.n_tiles_n = L.cout / L.bn;
+}
+
+// The tiles of the launches themselves: a one-agent launch waits layer by
+// layer, so choose_tiles; over several agents the layers flow.  A split
+// layer's tiles are always 64 wide, for the DSMEM exchange or for the four
+// slices of a tile side by side in one accumulator.
+void choose_launch_tiles(ConvLayer& L, int grid, int nb) {
+  pick_tile_batch(L, L.splits, grid, nb, L.splits > 1, nb > 1, &L);
   L.n_tiles_n = L.cout / L.bn;
 }
 
@@ -598,45 +608,15 @@ rtcc_status build_backbone(rtcc_ctx* c) {
       c->layers.push_back(L);
     }
   }
-  // fp32 workspace of the global-memory split-K reduction (used when a split
-  // layer cannot reduce through DSMEM): one per branch for its own launches,
-  // and one for the batched launches; deconvs never split
-  size_t ws_floats = 0, max_tiles = 0;
-  for (ConvLayer& L : c->layers) {
-    const int m_tiles = ((L.gw + conv_tile_w() - 1) / conv_tile_w()) *
-                        ((L.gh + conv_tile_h() - 1) / conv_tile_h());
-    if (L.kind == DECONV || L.splits < 1) L.splits = 1;
-    if (L.splits > 1) {
-      // the widest tile any batch size may pick: co / 32 tiles of 32 ... 128 columns
-      ws_floats = std::max(ws_floats, (size_t)L.splits * m_tiles * L.cout * conv_tile_m());
-      max_tiles = std::max(max_tiles, (size_t)m_tiles * (L.cout / 32));
-    }
-  }
-  c->splitk_cnt_bytes = max_tiles * sizeof(int);
-  for (int k = 0; k < K; ++k) {
-    Branch& b = c->br[k];
-    if (ws_floats) {
-      RS(dalloc(c, &b.splitk_ws, ws_floats * sizeof(float)));
-      RS(dalloc(c, &b.splitk_cnt, max_tiles * sizeof(int)));
-      CK(cudaMemset(b.splitk_cnt, 0, max_tiles * sizeof(int)));
-    }
-  }
-  if (ws_floats) {
-    RS(dalloc(c, &c->batch_ws, (size_t)K * ws_floats * sizeof(float)));
-    RS(dalloc(c, &c->batch_cnt, (size_t)K * max_tiles * sizeof(int)));
-    CK(cudaMemset(c->batch_cnt, 0, (size_t)K * max_tiles * sizeof(int)));
-  }
-  RS(dalloc(c, &c->batch_bar, (kMaxLayers + 1) * sizeof(unsigned)));
-  CK(cudaMemset(c->batch_bar, 0, (kMaxLayers + 1) * sizeof(unsigned)));
+  RS(dalloc(c, &c->batch_bar, kBarWords * sizeof(unsigned)));
+  CK(cudaMemset(c->batch_bar, 0, kBarWords * sizeof(unsigned)));
   c->wait_budget = (g.flags & RTCC_FLAG_SHORT_WAITS) ? 20000000LL : 2000000000LL;
   // launch parameters per batch size: the same K slices, the N tile and tile
   // height chosen for the batch
   for (int nb = 1; nb <= K; ++nb) {
     std::vector<ConvLayer> Lb = c->layers;
     for (ConvLayer& L : Lb) {
-      if (L.kind != DECONV) choose_tiles(L, grid, nb);
-      L.ws = c->batch_ws;
-      L.counters = c->batch_cnt;
+      if (L.kind != DECONV) choose_launch_tiles(L, grid, nb);
       if (conv_make_maps(L, c->bf16) != cudaSuccess) return RTCC_E_CUDA;
     }
     if (nb == 1) c->layers = Lb;                      // the maps of the one-agent tiles
@@ -649,8 +629,8 @@ rtcc_status build_backbone(rtcc_ctx* c) {
   c->launch_p = new (std::nothrow) BackboneParams;
   if (!c->launch_p) return RTCC_E_NOMEM;
   if (apart) {
-    RS(dalloc(c, &c->neck_bar, (kMaxLayers + 1) * sizeof(unsigned)));
-    CK(cudaMemset(c->neck_bar, 0, (kMaxLayers + 1) * sizeof(unsigned)));
+    RS(dalloc(c, &c->neck_bar, kBarWords * sizeof(unsigned)));
+    CK(cudaMemset(c->neck_bar, 0, kBarWords * sizeof(unsigned)));
     c->neck_p = new (std::nothrow) BackboneParams;
     if (!c->neck_p) return RTCC_E_NOMEM;
     if (backbone_fill(c->neck_layers, 1, c->neck_bar, c->d_err, nullptr, false, c->wait_budget, c->neck_p) !=
@@ -746,10 +726,6 @@ rtcc_status build_branch_params(rtcc_ctx* c, int k) {
   b.bb->stamps = b.stamps;
   b.bb->done_word = c->done_words + k;
   b.bb->stall = c->stall;
-  for (int l = 0; l < b.bb->n_layers; ++l) {
-    b.bb->L[l].ws = b.splitk_ws;
-    b.bb->L[l].counters = b.splitk_cnt;
-  }
   return RTCC_OK;
 }
 
@@ -1622,17 +1598,13 @@ rtcc_status rtcc_wait_detection(rtcc_ctx* c, int32_t timeout_ms, rtcc_box* out, 
   }
   if (hdr->err) {
     // A bounded device wait ran out.  The frame's kernels have all ended (the
-    // post-join waited for them); clear the error word and the split-K tile
-    // counters a kernel that wound down may have left, so the next frame
-    // starts clean.
+    // post-join waited for them); clear the error word and the counters a
+    // kernel that wound down may have left, so the next frame starts clean.
     for (int k = 0; k < c->K; ++k) cudaStreamSynchronize(c->br[k].st);
     cudaStreamSynchronize(c->bbst);
     cudaStreamSynchronize(c->post);
     CK(cudaMemset(c->d_err, 0, 16));
-    for (int k = 0; k < c->K; ++k)
-      if (c->br[k].splitk_cnt) CK(cudaMemset(c->br[k].splitk_cnt, 0, c->splitk_cnt_bytes));
-    if (c->batch_cnt) CK(cudaMemset(c->batch_cnt, 0, (size_t)c->K * c->splitk_cnt_bytes));
-    CK(cudaMemset(c->batch_bar, 0, (kMaxLayers + 1) * sizeof(unsigned)));
+    CK(cudaMemset(c->batch_bar, 0, kBarWords * sizeof(unsigned)));
     // the pillar passes' per-cell state and their image cells, as at allocation
     const size_t cells = (size_t)c->W * c->H;
     for (int k = 0; k < c->K; ++k) {

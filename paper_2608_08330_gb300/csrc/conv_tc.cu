@@ -15,25 +15,29 @@
 // stride-2 gather becomes a unit-stride box at a tap-dependent (channel half,
 // column, row parity, row) offset.  B (weights) is pre-packed K-major.
 //
-// The grid is one CTA per SM, co-resident (cooperative launch).  Work items of
-// a layer are dealt round-robin over the CTAs; each CTA counts itself in the
-// layer's arrival counter once its part of the layer is written, and a layer
-// whose input another CTA writes starts once the counter of the layer it
-// depends on shows every CTA (one counter per layer: a CTA with no work in
-// some layers runs ahead and must not be counted for a layer it has not
-// reached in the others' order).  Keeping the CTAs resident replaces
-// sixteen kernel boundaries (each a full drain and relaunch) by counter waits,
-// and lets the TMA/MMA pipeline and the tensor-memory allocation carry across
-// tiles and layers.
+// The grid is one CTA per SM, co-resident (cooperative launch).  Work items are
+// dealt round-robin over the CTAs, each layer going on where the one before
+// stopped (`rot`), so the CTAs' shares even out over the layers instead of the
+// same CTAs taking the last, partly filled round of each.  Items run
+// agent-major.  Each finished item counts itself in its (layer, agent)
+// counter; an item starts once every item of the same agent in the layer it
+// reads has been counted.  In a launch over several agents the other agents'
+// items lie in between, so a CTA flows from one layer into the next without
+// waiting for the slowest item of all agents; a one-agent launch waits layer
+// by layer.  Keeping the CTAs resident replaces sixteen kernel boundaries (each
+// a full drain and relaunch) by counter waits, and lets the TMA/MMA pipeline
+// and the tensor-memory allocation carry across tiles and layers.
 //
-// Roles (192 threads): warp 0 = TMA producer, warp 1 = tensor-memory owner and
-// MMA issuer, warps 2..5 = epilogue.  Tensor memory holds two 128-column
+// Roles (256 threads): warps 0, 6, 7 = TMA producers, warp 1 = tensor-memory
+// owner and MMA issuer, warps 2..5 = epilogue.  Tensor memory holds two 128-column
 // accumulators, so the epilogue of one tile overlaps the MMAs of the next.
 // The epilogue adds bias, applies ReLU, rounds to 16 bits and writes each
-// pixel's channels from registers (16-byte stores; a CTA's stores are then
-// published by one release-ordered count).  Split-K slices of a tile are
-// summed in slice order (through distributed shared memory, else global
-// memory), so results do not depend on timing.  Every
+// pixel's channels from registers (16-byte stores; an item's stores are then
+// published by one release-ordered count).  Split-K slices of a tile are summed
+// in slice order, on four CTAs through distributed shared memory or, where the
+// items of a launch do not fit the clustered grid, on one CTA in four
+// accumulators side by side: the same sums, and results do not depend on
+// timing.  Every
 // wait is bounded; one that runs out sets a bit in the error word and the CTA
 // winds down instead of hanging.
 #include <algorithm>
@@ -159,15 +163,16 @@ __device__ __forceinline__ bool grid_wait(const unsigned* ctr, unsigned target, 
 // memory clobber forces a reload) costs a constant-cache round trip each.
 struct LayerScalars {
   const float* bias;
-  float* ws;
-  int* counters;
   int kind, cin, cout, s, bn, bk, splits;
   int tiles_x, m_tiles, n_tiles, choff, wait_layers;
   int n_items, total_kb;
   int ncb_log2;            // log2(cin / bk): k-block kb = (tap << ncb_log2) + channel block
-  int dsm;                 // split-K slices reduced through distributed shared memory
-  int cta_lo, cta_hi;      // CTAs the items are dealt to
-  int wait_items;          // target of the awaited layer's counter
+  int dsm;                 // split-K slices on the ranks of a cluster, reduced through
+                           // distributed shared memory (one item per slice)
+  int stack;               // split-K slices this CTA accumulates side by side (1: no split)
+  int zs;                  // items per tile (the slices of a dsm layer, else 1)
+  int cta_lo, cta_hi, rot; // CTAs the items are dealt to, from CTA cta_lo + rot on
+  int wait_items;          // items per agent of the awaited layer (its counters' target)
   int halo;                // A from halo tiles; k-blocks chunk-major (kb = 9 chunk + tap)
   int tall;                // halo layers: tiles of TW x kTallTH pixels (two MMA row blocks
                            // sharing every weight box) instead of TW x TH
@@ -185,11 +190,11 @@ struct LayerScalars {
   int deconv_idx;
   int n_batch;
 };
-__device__ __forceinline__ LayerScalars layer_scalars(const LayerDesc& D, int n_batch) {
+__device__ __forceinline__ LayerScalars layer_scalars(const BackboneParams& P, int l, bool clustered) {
+  const LayerDesc& D = P.L[l];
+  const int n_batch = P.n_batch;
   LayerScalars S;
   S.bias = D.bias;
-  S.ws = D.ws;
-  S.counters = D.counters;
   S.kind = D.kind;
   S.cin = D.cin;
   S.cout = D.cout;
@@ -202,10 +207,19 @@ __device__ __forceinline__ LayerScalars layer_scalars(const LayerDesc& D, int n_
   S.n_tiles = D.n_tiles;
   S.choff = D.choff;
   S.wait_layers = D.wait_layers;
-  S.dsm = D.dsm;
+  // without the clusters the slices' exchange needs (a profiler's replay may
+  // drop them), a dsm layer's tiles become one item each
+  S.dsm = D.dsm && clustered;
+  S.zs = S.dsm ? D.splits : 1;
+  S.stack = S.dsm ? 1 : D.splits;
   S.cta_lo = D.cta_lo;
   S.cta_hi = D.cta_hi;
-  S.wait_items = D.wait_items;
+  S.rot = D.rot;
+  S.wait_items = 0;
+  if (D.wait_layers > 0) {
+    const LayerDesc& W = P.L[D.wait_layers - 1];
+    S.wait_items = W.m_tiles * W.n_tiles * (W.dsm && clustered ? W.splits : 1);
+  }
   S.halo = D.halo;
   S.tall = D.tall;
   S.tw_log2 = __ffs(D.tw) - 1;
@@ -213,7 +227,7 @@ __device__ __forceinline__ LayerScalars layer_scalars(const LayerDesc& D, int n_
   S.tr = D.tr;
   S.out = D.out;
   S.out_astride = D.out_astride;
-  S.ipa = D.ipa;
+  S.ipa = D.m_tiles * D.n_tiles * S.zs;
   S.deconv_idx = D.deconv_idx;
   S.n_batch = n_batch;
   S.ow = D.ow;
@@ -233,15 +247,18 @@ __device__ __forceinline__ LayerScalars layer_scalars(const LayerDesc& D, int n_
 __device__ __forceinline__ int first_item(const LayerScalars& S) {
   const int b = (int)blockIdx.x;
   if (b < S.cta_lo || b >= S.cta_hi) return -1;
-  return b - S.cta_lo < S.n_items ? b - S.cta_lo : -1;
+  int t = b - S.cta_lo - S.rot;
+  if (t < 0) t += S.cta_hi - S.cta_lo;
+  return t < S.n_items ? t : -1;
 }
 
 // Work item t of a layer -> (batch slot j, tile = (m tile, n tile), K slice
 // z), its agent, its tile origin and its k-block range [kb0, kb1).  Items
 // run agent-major, and within an agent the slice index runs fastest, so the
-// slices of a tile are consecutive items: with one item per CTA and a grid of
-// clusters of kMaxSplits CTAs they share a cluster, slice z on rank z (an
-// agent's item count is a multiple of the slice count).
+// slices of a dsm layer's tile are consecutive items: with one item per CTA, a
+// grid of clusters of kMaxSplits CTAs and `rot` a multiple of kMaxSplits they
+// share a cluster, slice z on rank z (an agent's item count is a multiple of
+// the slice count).
 struct Item {
   int x0, y0, n0, z, tile, kb0, kb1, slot, agent;
 };
@@ -250,15 +267,15 @@ __device__ __forceinline__ Item item_of(const LayerScalars& S, int t, const int*
   it.slot = t / S.ipa;
   it.agent = agents[it.slot];
   t -= it.slot * S.ipa;
-  it.z = t % S.splits;
-  it.tile = t / S.splits;
+  it.z = t % S.zs;
+  it.tile = t / S.zs;
   const int mt = it.tile % S.m_tiles;
   const int nt = it.tile / S.m_tiles;
   it.x0 = (mt % S.tiles_x) << S.tw_log2;
   it.y0 = (mt / S.tiles_x) * (S.tall ? kTallTH : S.th);
   it.n0 = nt * S.bn;
-  it.kb0 = (it.z * S.total_kb) / S.splits;
-  it.kb1 = ((it.z + 1) * S.total_kb) / S.splits;
+  it.kb0 = (it.z * S.total_kb) / S.zs;
+  it.kb1 = ((it.z + 1) * S.total_kb) / S.zs;
   return it;
 }
 
@@ -386,7 +403,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
   uint64_t* hfull = recvbar + 1;               // [kHalo] halo tiles
   uint64_t* hempty = hfull + kHalo;            // [kHalo]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(hempty + kHalo);
-  __shared__ int s_last;
   __shared__ float s_bias[2][128];             // bias of the tile in each accumulator
   __shared__ int s_agents[RTCC_MAX_AGENTS];    // the launch's agents (batch slot -> agent)
   const long long budget = P.wait_budget;
@@ -452,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
       unsigned stall = (P.stall && *P.stall != 0) ? 1u : 0u;
       for (int l = 0; l < P.n_layers && alive; ++l) {
         const LayerDesc& D = P.L[l];
-        const LayerScalars S = layer_scalars(D, P.n_batch);
+        const LayerScalars S = layer_scalars(P, l, clustered);
         const CUtensorMap* mapA = &D.mapA;
         const CUtensorMap* mapB = &D.mapB;
         const CUtensorMap* mapB1 = &D.mapB1;
@@ -491,15 +507,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
           pdl_wait();
           waited_pdl = true;
         }
-        if (S.wait_layers > 0) {
-          // every item of the layer this one reads has been stored
-          if (!grid_wait(&P.grid_bar[S.wait_layers - 1], (unsigned)S.wait_items + stall, budget)) {
-            atomicOr(P.err, ERR_WAIT_PRODUCER);
-            alive = false;
-            break;
+        // Every item of the same agent in the layer this one reads has been
+        // stored: waited for once per agent, before the first box of its input
+        // (with stamps every agent's, so that the layers' spans follow each
+        // other).
+        int ready = -1;                          // batch slot known to be ready
+        auto input_ready = [&](int slot) -> bool {
+          if (S.wait_layers == 0 || slot == ready) return true;
+          const int j0 = P.stamps ? 0 : slot, j1 = P.stamps ? P.n_batch : slot + 1;
+          for (int j = j0; j < j1; ++j) {
+            if (!grid_wait(&P.grid_bar[(S.wait_layers - 1) * RTCC_MAX_AGENTS + j],
+                           (unsigned)S.wait_items + stall, budget))
+              return false;
+            stall = 0;
           }
-          stall = 0;
+          ready = slot;
           fence_async_global();
+          return true;
+        };
+        if (!input_ready(I0.slot)) {
+          atomicOr(P.err, ERR_WAIT_PRODUCER);
+          alive = false;
+          break;
         }
         // Tap boxes and halo tiles share the A area: before it changes use,
         // the MMAs that read it must be done.  The issuer commits every stage
@@ -542,6 +571,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             if (!mbar_wait(&hempty[h], ((hk / kHalo) & 1) ^ 1, budget)) return false;
             const int i = k / nch, c = k - i * nch;
             const Item In = (i == 0) ? I0 : item_of(S, t0 + i * tstep, s_agents);
+            if (!input_ready(In.slot)) return false;
             mbar_arrive_expect_tx(&hfull[h], hbytes);
             load_halo(mapA, smem + h * kHaloSlot, &hfull[h], In, In.kb0 / 9 + c);
             return true;
@@ -581,6 +611,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
         } else {
           for (int t = t0; t < S.n_items && alive; t += tstep) {
             const Item I = (t == t0) ? I0 : item_of(S, t, s_agents);
+            if (!input_ready(I.slot)) {
+              atomicOr(P.err, ERR_WAIT_PRODUCER);
+              alive = false;
+              break;
+            }
             for (int kb = I.kb0; kb < I.kb1; ++kb, ++it) {
               if (it % kProducers != pid) continue;
               const int s = it % kStages;
@@ -616,7 +651,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
     bool alive = true;
     const uint32_t smem0 = smem_u32(smem);
     for (int l = 0; l < P.n_layers && alive; ++l) {
-      const LayerScalars S = layer_scalars(P.L[l], P.n_batch);
+      const LayerScalars S = layer_scalars(P, l, clustered);
       const uint32_t idesc = idesc_f16(BM, S.bn, std::is_same<T, __nv_bfloat16>::value);
       const bool bk64 = S.bk == 64;
       const uint32_t swz = bk64 ? 2u : 4u;            // 128B : 64B swizzle
@@ -647,6 +682,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
           // same weight box with the A rows TH halo rows further down.
           const bool tall = S.tall != 0;
           const int nch = (I.kb1 - I.kb0) / 9;
+          const int cps = nch / S.stack;                      // chunks per K slice
           const int km = S.kpb - 1;
           const uint32_t bstep = (uint32_t)(S.bn * 8);        // one weight box, 16-byte units
           for (int c = 0; c < nch && alive; ++c) {
@@ -658,15 +694,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             }
             ++hc;
             const uint32_t a_lo = (uint32_t)smem_desc(smem0 + h * kHaloSlot, kHaloW * 128, 2u);
-            const bool acc_in = c > 0;
+            // stacked K slices: 64 accumulator columns each
+            const int z = c / cps;
+            const bool acc_in = c > z * cps;
+            const uint32_t d_slice = d_tmem + (uint32_t)(z * 64);
             const bool ok =
-                tall ? (S.tr ? halo_chunk_mma<true, true>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km, bstep,
+                tall ? (S.tr ? halo_chunk_mma<true, true>(d_slice, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km, bstep,
                                                           acc_in, full, empty, it, leader, budget)
-                             : halo_chunk_mma<true, false>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
+                             : halo_chunk_mma<true, false>(d_slice, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
                                                            bstep, acc_in, full, empty, it, leader, budget))
-                     : (S.tr ? halo_chunk_mma<false, true>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
+                     : (S.tr ? halo_chunk_mma<false, true>(d_slice, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
                                                            bstep, acc_in, full, empty, it, leader, budget)
-                             : halo_chunk_mma<false, false>(d_tmem, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
+                             : halo_chunk_mma<false, false>(d_slice, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km,
                                                             bstep, acc_in, full, empty, it, leader, budget));
             if (!ok) {
               if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
@@ -677,7 +716,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             __syncwarp();
           }
         } else {
+          int z = 0, kz = I.kb0;                              // K slice (stacked) and its first k-block
           for (int kb = I.kb0; kb < I.kb1; ++kb, ++it) {
+            if (S.stack > 1 && kb == ((z + 1) * S.total_kb) / S.stack) {
+              ++z;
+              kz = kb;
+            }
             const int s = it % kStages;
             if (!mbar_wait_warp(&full[s], (it / kStages) & 1, budget)) {
               if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
@@ -686,8 +730,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             }
             tc_fence_after();
             if (leader) {
-              mma_kblock(d_tmem, a_lo0 + (uint32_t)(s * (kABytes >> 4)), a_hi,
-                         b_lo0 + (uint32_t)(s * (kBBytes >> 4)), b_hi, idesc, kb > I.kb0 ? 1u : 0u, bk64);
+              mma_kblock(d_tmem + (uint32_t)(z * 64), a_lo0 + (uint32_t)(s * (kABytes >> 4)), a_hi,
+                         b_lo0 + (uint32_t)(s * (kBBytes >> 4)), b_hi, idesc, kb > kz ? 1u : 0u, bk64);
               umma_commit(&empty[s]);
             }
             __syncwarp();
@@ -708,7 +752,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
     uint32_t tc = 0, dsm_phase = 0;
     bool alive = true;
     for (int l = 0; l < P.n_layers; ++l) {
-      const LayerScalars S = layer_scalars(P.L[l], P.n_batch);
+      const LayerScalars S = layer_scalars(P, l, clustered);
       const int t0 = first_item(S), tstep = S.cta_hi - S.cta_lo;
       if (t0 < 0) continue;                    // no items here: no count
       int mine = 0;
@@ -751,7 +795,29 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
         // (deconv) must have read the shared memory they came from
         if ((S.dsm && row == 0) || (S.kind == DECONV && deconv_storer(row, S.bn))) bulk_wait_read_all();
         epilogue_sync();
-        if (S.splits == 1) {
+        if (S.splits > 1 && !S.dsm) {
+          // stacked K slices: 16 columns of every slice at a time, summed in
+          // slice order
+          for (int c0 = 0; c0 < 64; c0 += 16) {
+            uint32_t r[kMaxSplits][16];
+#pragma unroll
+            for (int zz = 0; zz < kMaxSplits; ++zz)
+              if (zz < S.splits) tmem_ld16_issue(taddr + zz * 64 + c0, r[zz]);
+            tmem_ld_wait();
+            float sum[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[j] = 0.f;
+#pragma unroll
+            for (int zz = 0; zz < kMaxSplits; ++zz) {
+              if (zz < S.splits) {
+                tmem_reg_fence(r[zz]);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) sum[j] += __uint_as_float(r[zz][j]);
+              }
+            }
+            store16<T>(orow ? orow + c0 : nullptr, sum, bias + c0);
+          }
+        } else if (S.splits == 1) {
           // up to 64 columns per round: issue all TMEM loads, wait once; a
           // tall tile's lower row block (TH image rows further down) follows
           // from accumulator columns +128
@@ -789,7 +855,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
               }
             }
           }
-        } else if (S.dsm && clustered) {
+        } else {
           // The Sp = splits (2 or 4) K-slices of this 64-wide tile sit on Sp
           // consecutive ranks of this cluster of four, slice z on rank gb + z.
           // Reduce-scatter through distributed shared memory: slice z owns the
@@ -859,70 +925,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             // bias + ReLU, 16-bit, the owner's 16 channels of this row
             store16<T>(orow ? orow + z * CW + h * 16 : nullptr, sum, bias + z * CW + h * 16);
           }
-        } else {
-          // publish this slice's fp32 partial ([bn/4][BM][4] per (slice, tile),
-          // so a warp's float4 stores cover 512 contiguous bytes), then the
-          // last slice of the tile sums the slices in slice order (tiles of
-          // the batch's agents numbered slot-major)
-          const int tiles = S.n_batch * S.m_tiles * S.n_tiles;
-          const int tile_id = I.slot * S.m_tiles * S.n_tiles + I.tile;
-          float4* mine =
-              reinterpret_cast<float4*>(S.ws + (size_t)(I.z * tiles + tile_id) * BM * S.bn) + row;
-          for (int c0 = 0; c0 < S.bn; c0 += 16) {
-            float v[16];
-            tmem_ld16(taddr + c0, v);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              mine[(c0 / 4 + q) * BM] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          }
-          __threadfence();
-          epilogue_sync();
-          if (row == 0) {
-            const int old = atomicAdd(&S.counters[tile_id], 1);
-            s_last = (old == S.splits - 1);
-          }
-          epilogue_sync();
-          if (s_last != 0) {
-            __threadfence();
-            for (int c0 = 0; c0 < S.bn; c0 += 16) {
-              // all other slices' loads of this column group in flight at once
-              float4 f[kMaxSplits][4];
-#pragma unroll
-              for (int zz = 0; zz < kMaxSplits; ++zz) {
-                if (zz < S.splits && zz != I.z) {
-                  const float4* src =
-                      reinterpret_cast<const float4*>(S.ws + (size_t)(zz * tiles + tile_id) * BM * S.bn) +
-                      row;
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) f[zz][q] = __ldcg(src + (c0 / 4 + q) * BM);
-                }
-              }
-              float v[16];
-              tmem_ld16(taddr + c0, v);
-              float sum[16];
-#pragma unroll
-              for (int j = 0; j < 16; ++j) sum[j] = 0.f;
-#pragma unroll
-              for (int zz = 0; zz < kMaxSplits; ++zz) {
-                if (zz < S.splits) {
-                  if (zz == I.z) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) sum[j] += v[j];
-                  } else {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                      sum[4 * q] += f[zz][q].x;
-                      sum[4 * q + 1] += f[zz][q].y;
-                      sum[4 * q + 2] += f[zz][q].z;
-                      sum[4 * q + 3] += f[zz][q].w;
-                    }
-                  }
-                }
-              }
-              store16<T>(orow ? orow + c0 : nullptr, sum, bias + c0);
-            }
-            if (row == 0) S.counters[tile_id] = 0;     // ready for the next launch
-          }
         }
         // the accumulator has been read: hand it back to the MMA issuer
         tc_fence_before();
@@ -942,27 +944,39 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             tma_store_5d(mapC, stage + g * BM * 128, S.choff + g * 64, sx, I.x0, sy, I.y0);
             bulk_commit();
           }
-        }
-      }
-      // This CTA's items of layer l are stored: count them.  The epilogue
-      // threads' stores are ordered before the count by the barrier and the
-      // count's release semantics (cumulative over what the barrier made
-      // visible to this thread), so a consumer that acquires the counter
-      // sees them.  (With TMA stores, waiting for their completion and a
-      // full __threadfence here cost about a microsecond per layer.)
-      if (S.kind == DECONV && deconv_storer(row, S.bn)) {   // TMA stores: complete, then ordered
-        bulk_wait_all();
-        fence_async_global();
-      }
-      epilogue_sync();
-      if (row == 0) {
-        if (P.stamps) {
-          const unsigned before = atom_add_release_gpu(&P.grid_bar[l], (unsigned)mine);
-          // the CTA completing the layer's count stamps its end
-          if (before + (unsigned)mine == (unsigned)S.n_items) P.stamps[P.n_layers + l] = global_ns();
         } else {
-          red_add_release_gpu(&P.grid_bar[l], (unsigned)mine);
+          // The item is stored: count it for its agent.  The epilogue threads'
+          // stores are ordered before the count by the barrier and the count's
+          // release semantics (cumulative over what the barrier made visible
+          // to this thread), so a consumer that acquires the counter sees
+          // them.  (With TMA stores, waiting for their completion and a full
+          // __threadfence here cost about a microsecond per layer.)
+          epilogue_sync();
+          if (row == 0) {
+            unsigned* ctr = &P.grid_bar[l * RTCC_MAX_AGENTS + I.slot];
+            if (P.stamps) {
+              // an item that completes its agent's count stamps the layer's end so far
+              if (atom_add_release_gpu(ctr, 1u) + 1u == (unsigned)S.ipa)
+                atomicMax(&P.stamps[P.n_layers + l], global_ns());
+            } else {
+              red_add_release_gpu(ctr, 1u);
+            }
+          }
         }
+      }
+      // Deconvs: nothing in this launch reads them; the launch's end waits for
+      // their stores, and with stamps the layer's items are counted (in the
+      // first agent's word).
+      if (S.kind == DECONV) {
+        if (deconv_storer(row, S.bn)) {
+          bulk_wait_all();
+          fence_async_global();
+        }
+        epilogue_sync();
+        if (row == 0 && P.stamps &&
+            atom_add_release_gpu(&P.grid_bar[l * RTCC_MAX_AGENTS], (unsigned)mine) + (unsigned)mine ==
+                (unsigned)S.n_items)
+          atomicMax(&P.stamps[P.n_layers + l], global_ns());
       }
     }
   }
@@ -979,10 +993,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
   // launch's end to the host.
   if (threadIdx.x == 0) {
     __threadfence();
-    const unsigned old = atomicAdd(&P.grid_bar[kMaxLayers], 1u);
+    const unsigned old = atomicAdd(&P.grid_bar[kBarWords - 1], 1u);
     if (old == gridDim.x - 1) {
-      for (int l = 0; l < P.n_layers; ++l) P.grid_bar[l] = 0u;
-      P.grid_bar[kMaxLayers] = 0u;
+      for (int i = 0; i < P.n_layers * RTCC_MAX_AGENTS; ++i) P.grid_bar[i] = 0u;
+      P.grid_bar[kBarWords - 1] = 0u;
       if (P.done_word) {
         __threadfence_system();
         *P.done_word = 1;
@@ -1199,7 +1213,8 @@ cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, uns
         L.bn > 128 || L.bk > 64 || L.bn % 32)
       return cudaErrorInvalidValue;
     const int total_kb = (L.kind == DECONV ? 1 : 9) * (L.cin / L.bk);
-    if (L.splits < 1 || L.splits > kMaxSplits || L.splits > total_kb || (L.splits > 1 && (!L.ws || !L.counters)))
+    if (L.splits < 1 || L.splits > kMaxSplits || L.splits > total_kb ||
+        (L.splits > 1 && (L.bn != 64 || L.kind == DECONV)))
       return cudaErrorInvalidValue;
     LayerDesc& D = P->L[i];
     D.mapA = L.mapA;
@@ -1213,8 +1228,6 @@ cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, uns
       ++n_deconv;
     }
     D.bias = L.bias;
-    D.ws = L.ws;
-    D.counters = L.counters;
     D.kind = L.kind;
     D.cin = L.cin;
     D.cout = L.cout;
@@ -1236,7 +1249,6 @@ cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, uns
     D.wait_layers = L.wait_layers;
     D.out = L.out;
     D.out_astride = L.out_astride;
-    D.ipa = D.m_tiles * D.n_tiles * L.splits;
     D.ow = L.out_w;
     D.ldc = L.ldc;
     D.gw = gx;
@@ -1244,42 +1256,58 @@ cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, uns
     D.halo = conv_uses_halo(L) ? 1 : 0;
     // a split of a 64-wide tile into 2 or kMaxSplits slices, one item per
     // CTA, reduces its slices through distributed shared memory within a
-    // cluster of kMaxSplits CTAs
-    D.dsm = (L.kind != DECONV && (L.splits == 2 || L.splits == kMaxSplits) && L.bn == 64 && grid_cl > 0 &&
-             n_batch * D.ipa <= grid_cl)
+    // cluster of kMaxSplits CTAs; where the slices of a launch outnumber the
+    // CTAs, one CTA accumulates a tile's slices side by side instead (pp3,
+    // 3 agents: the deepest block's layers took 20 us each when the slices met
+    // in global memory)
+    D.dsm = ((L.splits == 2 || L.splits == kMaxSplits) && grid_cl > 0 &&
+             n_batch * D.m_tiles * D.n_tiles * L.splits <= grid_cl)
                 ? 1
                 : 0;
     any_dsm = any_dsm || D.dsm;
   }
   P->cluster = any_dsm ? kMaxSplits : 1;
   P->grid = any_dsm ? grid_cl : grid_sm;
-  // Item ranges.  Every layer's items are dealt round-robin over all CTAs,
-  // except the deconvs of the shallower blocks (those that do not read the
-  // deepest block): when the conv layers that can run at the same time as
-  // such a deconv (those after the layer it reads) leave at least 8 CTAs
-  // without items, those CTAs take the deconv, which then runs alongside the
-  // deeper conv blocks instead of after them (a CTA with no items in a layer
-  // skips it without waiting).  A layer waits for the items of the one layer
-  // it reads.
+  // Item ranges.  Every layer's items are dealt round-robin over all CTAs, each
+  // layer from the CTA after the one before it stopped at, except the deconvs
+  // of the shallower blocks (those that do not read the deepest block): when
+  // the conv layers that can run at the same time as such a deconv (those
+  // after the layer it reads) leave at least 8 CTAs without items, those CTAs
+  // take the deconv, which then runs alongside the deeper conv blocks instead
+  // of after them (a CTA with no items in a layer skips it without waiting).
+  // The idle CTAs then have to be the same in every layer, and they have to
+  // get through the deconv meanwhile: about 2.6 us an item against 8 us a
+  // layer (8 CTAs once took 106 us over a deconv of 378 items).
+  auto items_of = [&](const LayerDesc& D) { return n_batch * D.m_tiles * D.n_tiles * (D.dsm ? D.splits : 1); };
   int last_conv = -1;
   for (int i = 0; i < P->n_layers; ++i)
     if (P->L[i].kind != DECONV) last_conv = i;
+  bool beside = false;
   for (int i = 0; i < P->n_layers; ++i) {
     LayerDesc& D = P->L[i];
     D.cta_lo = 0;
     D.cta_hi = P->grid;
-    if (D.kind == DECONV && D.wait_layers >= 1 && D.wait_layers - 1 != last_conv) {
-      int conc_max = 0;                            // conv items beside this deconv
-      for (int j = D.wait_layers; j < P->n_layers; ++j)
-        if (P->L[j].kind != DECONV) conc_max = std::max(conc_max, n_batch * P->L[j].ipa);
-      if (P->grid - conc_max >= 8) D.cta_lo = conc_max;
-    }
+    D.rot = 0;
     if (D.wait_layers > P->n_layers || D.wait_layers > (int)i) return cudaErrorInvalidValue;
-    D.wait_items = 0;
-    if (D.wait_layers > 0) {
-      const LayerDesc& W = P->L[D.wait_layers - 1];
-      D.wait_items = n_batch * W.ipa;
+    if (D.kind == DECONV && D.wait_layers >= 1 && D.wait_layers - 1 != last_conv) {
+      int conc_max = 0, conc = 0;                  // conv items beside this deconv, their layers
+      for (int j = D.wait_layers; j < P->n_layers; ++j)
+        if (P->L[j].kind != DECONV) {
+          conc_max = std::max(conc_max, items_of(P->L[j]));
+          ++conc;
+        }
+      const int idle = P->grid - conc_max;
+      if (idle >= 8 && 5 * ((items_of(D) + idle - 1) / idle) <= 16 * conc) {
+        D.cta_lo = conc_max;
+        beside = true;
+      }
     }
+  }
+  for (int i = 0, next = 0; i < P->n_layers && !beside; ++i) {
+    LayerDesc& D = P->L[i];
+    if (D.dsm) next = (next + kMaxSplits - 1) / kMaxSplits * kMaxSplits % P->grid;   // slice z on rank z
+    D.rot = next;
+    next = (next + items_of(D)) % P->grid;
   }
   return cudaSuccess;
 }

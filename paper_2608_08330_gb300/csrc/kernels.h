@@ -144,8 +144,6 @@ struct ConvLayer {
                          // 8 pixels along H by 16 (tall: 32) along W
   int wide;              // tap-box convs without split-K: tiles of 16 x 8 pixels
   int wait_layers;       // this layer reads outputs of layers [0, wait_layers)
-  float* ws;             // split-K partials [batch][splits][m_tiles * n_tiles][128][bn] fp32
-  int* counters;         // split-K arrivals per tile [batch][m_tiles * n_tiles], zero-initialised
   const void* in;        // device [agent][in_h][in_w][cin]
   void* out;             // device [agent][out_h][out_w][ldc]
   const void* wpacked;   // device, K-major: conv [9][Cout][Cin]; deconv [s*s*Cout][Cin]
@@ -176,18 +174,18 @@ bool conv_shape_ok(const ConvLayer& L);
 // One layer of the persistent backbone kernel (kernel-parameter layout).
 constexpr int kMaxLayers = 20;
 constexpr int kMaxDeconv = 3;     // neck deconvs (one per block)
-constexpr int kMaxSplits = 4;     // split-K slices per tile (the reducing slice keeps one load per slice in flight)
+constexpr int kMaxSplits = 4;     // split-K slices per tile
+constexpr int kBarWords = kMaxLayers * RTCC_MAX_AGENTS + 1;   // counters of a backbone launch
 struct alignas(128) LayerDesc {   // CUtensorMap is 128-byte aligned
   CUtensorMap mapA, mapB, mapB1;
   const float* bias;
-  float* ws;
-  int* counters;
   int kind, cin, cout, s, bn, bk, splits;
   int tiles_x, m_tiles, n_tiles, choff;
   int wait_layers;
   int dsm;                       // split-K slices reduced through distributed shared memory
-  int cta_lo, cta_hi;            // the CTAs this layer's items are dealt to (round-robin)
-  int wait_items;                // items of layer wait_layers - 1 (its counter's target)
+                                 // (else side by side on one CTA)
+  int cta_lo, cta_hi;            // the CTAs this layer's items are dealt to (round-robin),
+  int rot;                       // from CTA cta_lo + rot on
   int halo;                      // 3x3 stride-1 with 64-channel k-blocks: A from halo tiles
   int tall;                      // halo layers: tiles two MMA row blocks high (see ConvLayer)
   int tw, th;                    // tile width and height (one MMA row block) in pixels
@@ -195,7 +193,6 @@ struct alignas(128) LayerDesc {   // CUtensorMap is 128-byte aligned
   void* out;                     // output [agent][out_h][ow][ldc], channels from choff
   long long out_astride;         // elements between agents in `out`
   int ow, ldc, gw, gh;           // output row length, pixel stride, tile grid extent
-  int ipa;                       // items per agent (m_tiles * n_tiles * splits)
   int deconv_idx;                // deconvs: index into BackboneParams::mapC
 };
 struct BackboneParams {
@@ -204,7 +201,7 @@ struct BackboneParams {
   int n_layers;
   int n_batch;                   // agents this launch runs
   int agents[RTCC_MAX_AGENTS];   // their indices, ascending (the agent coordinate of the maps)
-  unsigned* grid_bar;            // [kMaxLayers + 1] per-layer counts of finished items, then
+  unsigned* grid_bar;            // [kBarWords] finished items per layer and batch slot, then
                                  // the CTA exit count; zero before a launch (the last CTA to
                                  // leave zeroes them again)
   int* err;
@@ -221,7 +218,7 @@ struct BackboneParams {
 
 // Fill the kernel parameters of a backbone launch over `n_batch` agents from
 // the layer list (whose bn fields are the N tiles for that batch size);
-// grid_bar holds kMaxLayers + 1 counters.  The agent list is set by the
+// grid_bar holds kBarWords counters.  The agent list is set by the
 // caller (agents[0 .. n_batch)).
 cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, unsigned* grid_bar,
                           int* err, unsigned long long* stamps, bool allow_clusters,
