@@ -553,7 +553,9 @@ rtcc_status rtcc_test_unreachable_wait(struct rtcc_ctx* ctx);
  * Writes the kept boxes in order to host_out (room for n) and their number to
  * *n_out.  Boxes are rectangles in x-y: centre (x, y), length l along
  * (cos yaw, sin yaw), width w across it; z, h and score are carried along.
- * Synchronous; allocates and frees its own device scratch.
+ * Synchronous, and safe from several threads: each call takes a workspace of
+ * its own (36 KB of pinned and 50 KB of device memory), of which up to four stay
+ * allocated for later calls.
  */
 rtcc_status rtcc_nms(const rtcc_box* host_in, int32_t n, float iou, rtcc_box* host_out,
                      int32_t* n_out);

@@ -1871,54 +1871,4 @@ rtcc_status rtcc_test_unreachable_wait(rtcc_ctx* c) {
   return RTCC_OK;
 }
 
-rtcc_status rtcc_nms(const rtcc_box* host_in, int32_t n, float iou, rtcc_box* host_out,
-                     int32_t* n_out) {
-  if (n < 0 || n > kDecodeKeep || (n > 0 && (!host_in || !host_out)) || !n_out ||
-      !(iou >= 0.f && iou <= 1.f))
-    return RTCC_E_ARG;
-  const int mb = n > 0 ? n : 1;
-  // one scratch block: boxes in, count, ticket, error word, done word,
-  // result block (header + boxes), bitmask
-  const size_t in_b = (size_t)mb * sizeof(rtcc_box), res_b = sizeof(DetResultHeader) + in_b;
-  const size_t off_n = (in_b + 15) / 16 * 16, off_res = off_n + 64,
-               off_mask = off_res + (res_b + 15) / 16 * 16;
-  const size_t total = off_mask + nms_mask_words(mb) * sizeof(uint32_t);
-  uint8_t* d = nullptr;
-  if (cudaMalloc(&d, total) != cudaSuccess) return RTCC_E_NOMEM;
-  cudaStream_t st = nullptr;
-  rtcc_status r = RTCC_E_CUDA;
-  int* ints = reinterpret_cast<int*>(d + off_n);       // [0] n, [1] ticket, [2] err, [3] done
-  do {
-    if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) break;
-    if (cudaMemsetAsync(d + off_n, 0, 64, st) != cudaSuccess) break;
-    // bitmask scratch all ones (see the context's allocation)
-    if (cudaMemsetAsync(d + off_mask, 0xFF, nms_mask_words(mb) * sizeof(uint32_t), st) != cudaSuccess) break;
-    if (n > 0 && cudaMemcpyAsync(d, host_in, in_b, cudaMemcpyHostToDevice, st) != cudaSuccess) break;
-    if (cudaMemcpyAsync(ints, &n, sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess) break;
-    NmsArgs a{};
-    a.in = reinterpret_cast<const rtcc_box*>(d);
-    a.n_in = ints;
-    a.ticket = reinterpret_cast<unsigned*>(ints + 1);
-    a.err = ints + 2;
-    a.done = ints + 3;
-    a.mask = reinterpret_cast<uint32_t*>(d + off_mask);
-    a.max_boxes = mb;
-    a.iou = iou;
-    a.out = d + off_res;
-    if (launch_nms(a, st) != cudaSuccess) break;
-    DetResultHeader h{};
-    if (cudaMemcpyAsync(&h, d + off_res, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess) break;
-    if (cudaStreamSynchronize(st) != cudaSuccess) break;
-    const int k = std::max(0, std::min(h.n_boxes, n));
-    if (k > 0 && cudaMemcpy(host_out, d + off_res + sizeof(DetResultHeader), (size_t)k * sizeof(rtcc_box),
-                            cudaMemcpyDeviceToHost) != cudaSuccess)
-      break;
-    *n_out = k;
-    r = RTCC_OK;
-  } while (false);
-  if (st) cudaStreamDestroy(st);
-  cudaFree(d);
-  return r;
-}
-
 }  // extern "C"

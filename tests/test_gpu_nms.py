@@ -2,6 +2,7 @@
 rule, on constructed box sets: ragged and full 32-box chunks, the largest
 list (512), duplicates, disjoint sets, suppression chains, and thresholds 0
 and 1."""
+import concurrent.futures as cf
 import math
 
 import numpy as np
@@ -62,3 +63,20 @@ def test_nms_edge_cases(R):
     assert R.rtcc_nms(crowd, 1.0)["anchor"].tolist() == list(range(128))
     out = R.rtcc_nms(crowd, 0.0)                         # any overlap suppresses
     U.check_nms(crowd, out, 0.0)
+
+
+def test_nms_threads_and_shrinking_lists(R):
+    """Calls from more threads than workspaces stay allocated, each with lists
+    of changing length: every call sees its own boxes only."""
+    lists = [_crowd(n, 40 + i) for i, n in enumerate([512, 1, 65, 300, 32, 7, 511, 128])]
+    want = [R.rtcc_nms(b, 0.2) for b in lists]
+    for b, out in zip(lists, want):
+        U.check_nms(b, out, 0.2)
+
+    def turn(t):
+        return [(i, R.rtcc_nms(lists[i], 0.2)) for r in range(12) for i in [(t + r) % len(lists)]]
+
+    with cf.ThreadPoolExecutor(8) as ex:
+        for got in ex.map(turn, range(8)):
+            for i, out in got:
+                assert out.tobytes() == want[i].tobytes()
