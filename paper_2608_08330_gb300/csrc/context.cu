@@ -121,6 +121,7 @@ struct rtcc_ctx {
                                       // CTA of branch k's own backbone launch (k) or of
                                       // batched launch j (RTCC_MAX_AGENTS + j)
   int inflight = -1;                  // done word of the last backbone launched, -1 none
+  cudaEvent_t bb_ev = nullptr;        // event behind the last backbone launched
   int n_launches = 0;                 // backbone launches this frame
   int launch_size[RTCC_MAX_AGENTS] = {};
   int launch_word[RTCC_MAX_AGENTS] = {};
@@ -1100,9 +1101,12 @@ rtcc_status init_impl(rtcc_ctx* c, const float* weights) {
   for (int k = 0; k < c->K; ++k) RS(capture_branch(c, k));
   RS(capture_post(c));
   // warm-up: every graph once on empty payloads (pays first-launch costs),
-  // and one batched launch of every batch size
-  for (int k = 0; k < c->K; ++k) CK(cudaGraphLaunch(c->br[k].exec, c->br[k].st));
-  for (int k = 0; k < c->K; ++k) CK(cudaGraphLaunch(c->br[k].exec_host, c->br[k].st));
+  // and one batched launch of every batch size; one backbone at a time
+  for (int k = 0; k < c->K; ++k) {
+    CK(cudaGraphLaunch(c->br[k].exec, c->br[k].st));
+    CK(cudaGraphLaunch(c->br[k].exec_host, c->br[k].st));
+    CK(cudaStreamSynchronize(c->br[k].st));
+  }
   for (int k = 0; k < c->K; ++k) CK(cudaGraphLaunch(c->br[k].pill, c->br[k].st));
   for (int k = 0; k < c->K; ++k) CK(cudaStreamSynchronize(c->br[k].st));
   for (int n = 2; n <= c->K; ++n) {
@@ -1155,16 +1159,29 @@ void note_dispatch(rtcc_ctx* c, int k) {
   if (c->info.n_dispatched < RTCC_MAX_AGENTS) c->info.dispatch_order[c->info.n_dispatched++] = k;
 }
 
-void note_launch(rtcc_ctx* c, int word, int size) {
+void note_launch(rtcc_ctx* c, int word, int size, cudaEvent_t ev) {
   if (c->n_launches < RTCC_MAX_AGENTS) {
     c->launch_size[c->n_launches] = size;
     c->launch_word[c->n_launches] = word;
   }
   ++c->n_launches;
   c->inflight = word;
+  c->bb_ev = ev;
 }
 
-// Branch k released alone: pillar chain and its own backbone (one graph).
+bool backbone_busy(const rtcc_ctx* c) { return c->inflight >= 0 && c->done_words[c->inflight] == 0; }
+
+// Two backbones must never share the GPU: each needs all of its CTAs resident
+// (they wait for each other's items), and two that each hold part of the SMs
+// would wait until their bound.  A backbone launched while another runs goes
+// behind that one's event, whatever their streams.
+rtcc_status after_running_backbone(rtcc_ctx* c, cudaStream_t st) {
+  if (backbone_busy(c)) CK(cudaStreamWaitEvent(st, c->bb_ev, 0));
+  return RTCC_OK;
+}
+
+// Branch k released alone, no backbone running: pillar chain and its own
+// backbone (one graph).
 // Called with the context mutex held, as are the launches below.
 rtcc_status launch_full(rtcc_ctx* c, int k) {
   Branch& b = c->br[k];
@@ -1177,7 +1194,7 @@ rtcc_status launch_full(rtcc_ctx* c, int k) {
   b.stamp_src = k;
   b.launch_idx = c->n_launches;
   b.full_graph = true;
-  note_launch(c, k, 1);
+  note_launch(c, k, 1, b.done);
   note_dispatch(c, k);
   return RTCC_OK;
 }
@@ -1208,6 +1225,7 @@ rtcc_status launch_batch(rtcc_ctx* c) {
   const int n = (int)ag.size();
   if (n == 1) {
     Branch& b = c->br[ag[0]];
+    RS(after_running_backbone(c, b.st));
     c->done_words[ag[0]] = 0;
     if (tl) CK(cudaEventRecord(b.ev_bb0, b.st));
     CK(launch_backbone(*b.bb, c->bf16, b.st));
@@ -1216,7 +1234,7 @@ rtcc_status launch_batch(rtcc_ctx* c) {
     b.feat_ev = b.done;
     b.stamp_src = ag[0];
     b.launch_idx = c->n_launches;
-    note_launch(c, ag[0], 1);
+    note_launch(c, ag[0], 1, b.done);
     return RTCC_OK;
   }
   const int j = std::min(c->n_launches, RTCC_MAX_AGENTS - 1);
@@ -1228,6 +1246,7 @@ rtcc_status launch_batch(rtcc_ctx* c) {
   P.done_word = c->done_words + word;
   P.stall = c->stall;
   for (int k : ag) CK(cudaStreamWaitEvent(c->bbst, c->br[k].pill_done, 0));
+  RS(after_running_backbone(c, c->bbst));
   c->done_words[word] = 0;
   if (tl) CK(cudaEventRecord(c->batch_t0[j], c->bbst));
   CK(launch_backbone(P, c->bf16, c->bbst));
@@ -1238,11 +1257,9 @@ rtcc_status launch_batch(rtcc_ctx* c) {
     c->br[k].stamp_src = ag[0];
     c->br[k].launch_idx = c->n_launches;
   }
-  note_launch(c, word, n);
+  note_launch(c, word, n, c->batch_ev[j]);
   return RTCC_OK;
 }
-
-bool backbone_busy(const rtcc_ctx* c) { return c->inflight >= 0 && c->done_words[c->inflight] == 0; }
 
 rtcc_status launch_post(rtcc_ctx* c) {
   // the presence flags are set on the device by the branches that ran (their
@@ -1276,7 +1293,14 @@ rtcc_status after_event(rtcc_ctx* c, const std::vector<int>& released, double t_
   const bool batching = (c->cfg.flags & RTCC_FLAG_NO_BATCH) == 0;
   const bool last = c->ctrl.join_ready();
   if (!batching) {
-    for (int k : released) RS(launch_full(c, k));
+    for (int k : released) {
+      if (backbone_busy(c)) {
+        RS(launch_pill(c, k));
+        RS(launch_batch(c));
+      } else {
+        RS(launch_full(c, k));
+      }
+    }
   } else if (released.size() == 1 && last && c->pending.empty() && !backbone_busy(c)) {
     RS(launch_full(c, released[0]));
   } else if (!released.empty()) {
