@@ -170,7 +170,7 @@ struct LayerScalars {
   int dsm;                 // split-K slices on the ranks of a cluster, reduced through
                            // distributed shared memory (one item per slice)
   int stack;               // split-K slices this CTA accumulates side by side (1: no split)
-  int zs;                  // items per tile (the slices of a dsm layer, else 1)
+  int zs, zs_log2;         // items per tile (the slices of a dsm layer, else 1)
   int cta_lo, cta_hi, rot; // CTAs the items are dealt to, from CTA cta_lo + rot on
   int wait_items;          // items per agent of the awaited layer (its counters' target)
   int halo;                // A from halo tiles; k-blocks chunk-major (kb = 9 chunk + tap)
@@ -187,6 +187,7 @@ struct LayerScalars {
   long long out_astride;   // elements between agents in out
   int ow, ldc, gw, gh;     // output row length (pixels), pixel stride (channels), tile grid extent
   int ipa;                 // items per agent
+  FastDiv div_ipa, div_mt, div_tx;
   int deconv_idx;
   int n_batch;
 };
@@ -211,6 +212,7 @@ __device__ __forceinline__ LayerScalars layer_scalars(const BackboneParams& P, i
   // drop them), a dsm layer's tiles become one item each
   S.dsm = D.dsm && clustered;
   S.zs = S.dsm ? D.splits : 1;
+  S.zs_log2 = __ffs(S.zs) - 1;
   S.stack = S.dsm ? 1 : D.splits;
   S.cta_lo = D.cta_lo;
   S.cta_hi = D.cta_hi;
@@ -228,6 +230,9 @@ __device__ __forceinline__ LayerScalars layer_scalars(const BackboneParams& P, i
   S.out = D.out;
   S.out_astride = D.out_astride;
   S.ipa = D.m_tiles * D.n_tiles * S.zs;
+  S.div_ipa = D.div_ipa[S.dsm];
+  S.div_mt = D.div_mt;
+  S.div_tx = D.div_tx;
   S.deconv_idx = D.deconv_idx;
   S.n_batch = n_batch;
   S.ow = D.ow;
@@ -252,46 +257,49 @@ __device__ __forceinline__ int first_item(const LayerScalars& S) {
   return t < S.n_items ? t : -1;
 }
 
+// The k-blocks [*kb0, *kb1) of K slice z.
+__device__ __forceinline__ void slice_kbs(const LayerScalars& S, int z, int* kb0, int* kb1) {
+  *kb0 = (z * S.total_kb) >> S.zs_log2;
+  *kb1 = ((z + 1) * S.total_kb) >> S.zs_log2;
+}
+
 // Work item t of a layer -> (batch slot j, tile = (m tile, n tile), K slice
 // z), its agent, its tile origin and its k-block range [kb0, kb1).  Items
 // run agent-major, and within an agent the slice index runs fastest, so the
 // slices of a dsm layer's tile are consecutive items: with one item per CTA, a
 // grid of clusters of kMaxSplits CTAs and `rot` a multiple of kMaxSplits they
 // share a cluster, slice z on rank z (an agent's item count is a multiple of
-// the slice count).
+// the slice count).  The divisions are multiplications (FastDiv): as integer
+// divisions they took 1500 to 2000 clocks an item, in which the MMA warp issued
+// nothing.
 struct Item {
   int x0, y0, n0, z, tile, kb0, kb1, slot, agent;
 };
 __device__ __forceinline__ Item item_of(const LayerScalars& S, int t, const int* agents) {
   Item it;
-  it.slot = t / S.ipa;
+  it.slot = (int)quotient(S.div_ipa, (uint32_t)t);
   it.agent = agents[it.slot];
   t -= it.slot * S.ipa;
-  it.z = t % S.zs;
-  it.tile = t / S.zs;
-  const int mt = it.tile % S.m_tiles;
-  const int nt = it.tile / S.m_tiles;
-  it.x0 = (mt % S.tiles_x) << S.tw_log2;
-  it.y0 = (mt / S.tiles_x) * (S.tall ? kTallTH : S.th);
+  it.z = t & (S.zs - 1);
+  it.tile = t >> S.zs_log2;
+  const int nt = (int)quotient(S.div_mt, (uint32_t)it.tile);
+  const int mt = it.tile - nt * S.m_tiles;
+  const int ty = (int)quotient(S.div_tx, (uint32_t)mt);
+  it.x0 = (mt - ty * S.tiles_x) << S.tw_log2;
+  it.y0 = ty * (S.tall ? kTallTH : S.th);
   it.n0 = nt * S.bn;
-  it.kb0 = (it.z * S.total_kb) / S.zs;
-  it.kb1 = ((it.z + 1) * S.total_kb) / S.zs;
+  slice_kbs(S, it.z, &it.kb0, &it.kb1);
   return it;
 }
 
-// Pipeline stages of an item and the k-blocks [*k0, *k0 + *n) of its stage j.
-// Tap-box layers: one k-block per stage.  Halo layers: the item holds whole
-// 64-channel chunks, each split into spc stages of up to kpb taps.
+// Pipeline stages of an item.  Tap-box layers: one k-block per stage.  Halo
+// layers: the item holds whole 64-channel chunks, each split into spc stages
+// of up to kpb taps; stage_kbs: the k-blocks [*k0, *k0 + *n) of stage q of
+// chunk c.
 __device__ __forceinline__ int item_stages(const LayerScalars& S, const Item& I) {
   return S.halo ? (I.kb1 - I.kb0) / 9 * S.spc : I.kb1 - I.kb0;
 }
-__device__ __forceinline__ void stage_kbs(const LayerScalars& S, const Item& I, int j, int* k0, int* n) {
-  if (!S.halo) {
-    *k0 = I.kb0 + j;
-    *n = 1;
-    return;
-  }
-  const int c = j / S.spc, q = j - c * S.spc;
+__device__ __forceinline__ void stage_kbs(const LayerScalars& S, const Item& I, int c, int q, int* k0, int* n) {
   *k0 = I.kb0 + 9 * c + q * S.kpb;
   *n = min(S.kpb, 9 - q * S.kpb);
 }
@@ -488,8 +496,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
         const Item I0 = item_of(S, t0, s_agents);
         int npre = item_stages(S, I0);
         if (npre > kStages) npre = kStages;
-        for (int j = 0; j < npre; ++j) {
+        for (int j = 0, c = 0, q = 0; j < npre; ++j) {
           const uint32_t u = it + j;
+          const int jc = c, jq = q;              // a halo layer's chunk, stage in it
+          if (S.halo && ++q == S.spc) {
+            q = 0;
+            ++c;
+          }
           if (u % kProducers != pid) continue;
           const int s = u % kStages;
           if (!mbar_wait(&empty[s], ((u / kStages) & 1) ^ 1, budget)) {
@@ -497,8 +510,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             alive = false;
             break;
           }
-          int k0, n;
-          stage_kbs(S, I0, j, &k0, &n);
+          int k0 = I0.kb0 + j, n = 1;
+          if (S.halo) stage_kbs(S, I0, jc, jq, &k0, &n);
           mbar_arrive_expect_tx(&full[s], S.halo ? bbox * n : bytes);
           load_b(S, (S.halo && n < S.kpb) ? mapB1 : mapB, smem + kBOff + s * kBBytes, &full[s], I0, k0);
         }
@@ -558,25 +571,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
           // thread: that thread has just seen the release of the stage 5
           // earlier, so chunk k - 1 is done (tile k + 1's slot is free) and
           // the tile has a chunk of MMAs to land.
-          const int nch = (I0.kb1 - I0.kb0) / 9;       // chunks per item (the same for all)
-          const int n_halos = ((S.n_items - 1 - t0) / tstep + 1) * nch;
+          const int nch_log2 = S.ncb_log2 - S.zs_log2;
+          const int nch = 1 << nch_log2;               // chunks per item (the same for all)
           const uint32_t hbytes = S.tall ? (uint32_t)kHaloBytesTall : (uint32_t)kHaloBytes;
           const int trig = S.spc < 5 ? S.spc - 1 : 4;
           const uint32_t hc0 = hc;
-          // tile k of this layer (the threads take turns, so each works out
-          // the tile's item itself)
-          auto issue_halo = [&](int k) -> bool {
+          // tile k of this layer: chunk c of item In
+          auto issue_halo = [&](int k, const Item& In, int c) -> bool {
             const uint32_t hk = hc0 + (uint32_t)k;
             const int h = hk % kHalo;
             if (!mbar_wait(&hempty[h], ((hk / kHalo) & 1) ^ 1, budget)) return false;
-            const int i = k / nch, c = k - i * nch;
-            const Item In = (i == 0) ? I0 : item_of(S, t0 + i * tstep, s_agents);
             if (!input_ready(In.slot)) return false;
             mbar_arrive_expect_tx(&hfull[h], hbytes);
             load_halo(mapA, smem + h * kHaloSlot, &hfull[h], In, In.kb0 / 9 + c);
             return true;
           };
-          if (it % kProducers == pid && !issue_halo(0)) {
+          if (it % kProducers == pid && !issue_halo(0, I0, 0)) {
             atomicOr(P.err, ERR_WAIT_PRODUCER);
             break;
           }
@@ -586,10 +596,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             for (int c = 0; c < nch && alive; ++c, ++k) {
               for (int q = 0; q < S.spc && alive; ++q, ++it) {
                 if (it % kProducers != pid) continue;
-                const int j = c * S.spc + q;
-                if (!(t == t0 && j < npre)) {           // weights not already in flight
+                if (!(t == t0 && c * S.spc + q < npre)) {   // weights not already in flight
                   int k0, n;
-                  stage_kbs(S, I, j, &k0, &n);
+                  stage_kbs(S, I, c, q, &k0, &n);
                   const int s = it % kStages;
                   if (!mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, budget)) {
                     atomicOr(P.err, ERR_WAIT_PRODUCER);
@@ -599,15 +608,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
                   mbar_arrive_expect_tx(&full[s], bbox * n);
                   load_b(S, n < S.kpb ? mapB1 : mapB, smem + kBOff + s * kBBytes, &full[s], I, k0);
                 }
-                if (q == trig && k + 1 < n_halos && !issue_halo(k + 1)) {
-                  atomicOr(P.err, ERR_WAIT_PRODUCER);
-                  alive = false;
-                  break;
+                if (q == trig) {
+                  // the next tile, of this item or the next
+                  bool ok = true;
+                  if (c + 1 < nch)
+                    ok = issue_halo(k + 1, I, c + 1);
+                  else if (t + tstep < S.n_items)
+                    ok = issue_halo(k + 1, item_of(S, t + tstep, s_agents), 0);
+                  if (!ok) {
+                    atomicOr(P.err, ERR_WAIT_PRODUCER);
+                    alive = false;
+                    break;
+                  }
                 }
               }
             }
           }
-          hc = hc0 + (uint32_t)n_halos;
+          hc = hc0 + (uint32_t)k;
         } else {
           for (int t = t0; t < S.n_items && alive; t += tstep) {
             const Item I = (t == t0) ? I0 : item_of(S, t, s_agents);
@@ -664,7 +681,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
       const uint32_t a_hi_halo = (uint32_t)(smem_desc(smem0, kHaloW * 128, 2u) >> 32);
       const int t0 = first_item(S), tstep = S.cta_hi - S.cta_lo;
       for (int t = t0; t >= 0 && t < S.n_items && alive; t += tstep, ++tc) {
-        const Item I = item_of(S, t, s_agents);
+        int kb0, kb1;                              // all that the MMAs need of the item
+        slice_kbs(S, t & (S.zs - 1), &kb0, &kb1);
         const int acc = tc & 1;
         if (!mbar_wait_warp(&accempty[acc], ((tc >> 1) & 1) ^ 1, budget)) {
           if (lane == 0) atomicOr(P.err, ERR_WAIT_MMA);
@@ -681,8 +699,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
           // tall tile's lower row block (accumulator columns +128) takes the
           // same weight box with the A rows TH halo rows further down.
           const bool tall = S.tall != 0;
-          const int nch = (I.kb1 - I.kb0) / 9;
-          const int cps = nch / S.stack;                      // chunks per K slice
+          const int nch_log2 = S.ncb_log2 - S.zs_log2;
+          const int nch = 1 << nch_log2;
+          const int cps_log2 = nch_log2 - (__ffs(S.stack) - 1);   // chunks per K slice
           const int km = S.kpb - 1;
           const uint32_t bstep = (uint32_t)(S.bn * 8);        // one weight box, 16-byte units
           for (int c = 0; c < nch && alive; ++c) {
@@ -695,8 +714,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             ++hc;
             const uint32_t a_lo = (uint32_t)smem_desc(smem0 + h * kHaloSlot, kHaloW * 128, 2u);
             // stacked K slices: 64 accumulator columns each
-            const int z = c / cps;
-            const bool acc_in = c > z * cps;
+            const int z = c >> cps_log2;
+            const bool acc_in = c > (z << cps_log2);
             const uint32_t d_slice = d_tmem + (uint32_t)(z * 64);
             const bool ok =
                 tall ? (S.tr ? halo_chunk_mma<true, true>(d_slice, a_lo, a_hi_halo, b_lo0, b_hi, idesc, km, bstep,
@@ -716,9 +735,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
             __syncwarp();
           }
         } else {
-          int z = 0, kz = I.kb0;                              // K slice (stacked) and its first k-block
-          for (int kb = I.kb0; kb < I.kb1; ++kb, ++it) {
-            if (S.stack > 1 && kb == ((z + 1) * S.total_kb) / S.stack) {
+          int z = 0, kz = kb0;                                // K slice (stacked) and its first k-block
+          const int stack_log2 = __ffs(S.stack) - 1;
+          for (int kb = kb0; kb < kb1; ++kb, ++it) {
+            if (S.stack > 1 && kb == ((z + 1) * S.total_kb) >> stack_log2) {
               ++z;
               kz = kb;
             }
@@ -1213,7 +1233,7 @@ cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, uns
         L.bn > 128 || L.bk > 64 || L.bn % 32)
       return cudaErrorInvalidValue;
     const int total_kb = (L.kind == DECONV ? 1 : 9) * (L.cin / L.bk);
-    if (L.splits < 1 || L.splits > kMaxSplits || L.splits > total_kb ||
+    if (L.splits < 1 || L.splits > kMaxSplits || (L.splits & (L.splits - 1)) || L.splits > total_kb ||
         (L.splits > 1 && (L.bn != 64 || L.kind == DECONV)))
       return cudaErrorInvalidValue;
     LayerDesc& D = P->L[i];
@@ -1265,6 +1285,10 @@ cudaError_t backbone_fill(const std::vector<ConvLayer>& layers, int n_batch, uns
                 ? 1
                 : 0;
     any_dsm = any_dsm || D.dsm;
+    D.div_ipa[0] = fast_div((uint32_t)(D.m_tiles * D.n_tiles));
+    D.div_ipa[1] = fast_div((uint32_t)(D.m_tiles * D.n_tiles * D.splits));
+    D.div_mt = fast_div((uint32_t)D.m_tiles);
+    D.div_tx = fast_div((uint32_t)D.tiles_x);
   }
   P->cluster = any_dsm ? kMaxSplits : 1;
   P->grid = any_dsm ? grid_cl : grid_sm;

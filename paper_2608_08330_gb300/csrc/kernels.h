@@ -176,6 +176,23 @@ constexpr int kMaxLayers = 20;
 constexpr int kMaxDeconv = 3;     // neck deconvs (one per block)
 constexpr int kMaxSplits = 4;     // split-K slices per tile
 constexpr int kBarWords = kMaxLayers * RTCC_MAX_AGENTS + 1;   // counters of a backbone launch
+// Division by a divisor known on the host: n / d = floor(n * m / 2^64) with
+// m = ceil(2^64 / d), exact for every 32-bit n (m = 0 stands for d = 1).
+struct FastDiv {
+  uint64_t m;
+  uint32_t d;
+};
+inline FastDiv fast_div(uint32_t d) {
+  FastDiv f;
+  f.d = d > 0 ? d : 1;
+  f.m = f.d == 1 ? 0 : ~uint64_t(0) / f.d + 1;
+  return f;
+}
+__host__ __device__ inline uint32_t quotient(const FastDiv& f, uint32_t n) {
+  if (f.m == 0) return n;
+  const uint64_t lo = (uint64_t)n * (uint32_t)f.m, hi = (uint64_t)n * (uint32_t)(f.m >> 32);
+  return (uint32_t)((hi + (lo >> 32)) >> 32);
+}
 struct alignas(128) LayerDesc {   // CUtensorMap is 128-byte aligned
   CUtensorMap mapA, mapB, mapB1;
   const float* bias;
@@ -194,6 +211,8 @@ struct alignas(128) LayerDesc {   // CUtensorMap is 128-byte aligned
   long long out_astride;         // elements between agents in `out`
   int ow, ldc, gw, gh;           // output row length, pixel stride, tile grid extent
   int deconv_idx;                // deconvs: index into BackboneParams::mapC
+  FastDiv div_ipa[2];            // by the items per agent without and with dsm slices
+  FastDiv div_mt, div_tx;        // by m_tiles, tiles_x
 };
 struct BackboneParams {
   LayerDesc L[kMaxLayers];
