@@ -26,6 +26,11 @@ template <> struct Store<__half> {
     __half2 h = *reinterpret_cast<__half2*>(&u);
     return __half22float2(h);
   }
+  // two packed values: +0 for every non-positive one and for NaN, as relu_f
+  static __device__ __forceinline__ uint32_t relu2(uint32_t u) {
+    __half2 h = __hmax2(*reinterpret_cast<__half2*>(&u), __half2(__ushort_as_half(0), __ushort_as_half(0)));
+    return *reinterpret_cast<uint32_t*>(&h);
+  }
 };
 template <> struct Store<__nv_bfloat16> {
   static __device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
@@ -37,6 +42,11 @@ template <> struct Store<__nv_bfloat16> {
   static __device__ __forceinline__ float2 unpack2(uint32_t u) {
     __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&u);
     return __bfloat1622float2(h);
+  }
+  static __device__ __forceinline__ uint32_t relu2(uint32_t u) {
+    __nv_bfloat162 h = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&u),
+                               __nv_bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0)));
+    return *reinterpret_cast<uint32_t*>(&h);
   }
 };
 
@@ -446,6 +456,13 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16
       : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr));
+}
+
 // Wait for every TMEM load this thread has issued.
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -453,6 +470,10 @@ __device__ __forceinline__ void tmem_ld_wait() {
 
 // Ties the registers of an issued TMEM load to a point after tmem_ld_wait():
 // an empty asm that reads and writes them, so no use is scheduled earlier.
+__device__ __forceinline__ void tmem_reg_fence(uint32_t (&r)[8]) {
+  asm volatile(""
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+}
 __device__ __forceinline__ void tmem_reg_fence(uint32_t (&r)[16]) {
   asm volatile(""
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),

@@ -96,9 +96,9 @@ struct rtcc_ctx {
   // RTCC_FLAG_MULTISCALE: the branches end at their blocks; the post-join
   // fuses each block's map across the agents, then runs the neck once
   bool ms = false;
-  // Max fusion or multi-scale: the post-join runs the neck, the max and the
-  // head in one kernel over the blocks' outputs (neck_head.cu), and the
-  // feature maps are computed only when they are read back
+  // The post-join runs the neck, the fusion and the head in one kernel over
+  // the blocks' outputs (neck_head.cu), and the feature maps (single-scale
+  // attention: the fused map too) are computed only when they are read back
   bool fused_neck = false;
   void* fblk[RTCC_MAX_BLOCKS] = {};   // fused block maps [H_b][W_b][C_b]
   void* neck_out = nullptr;           // neck of the fused blocks [H'][W'][C_feat]
@@ -106,6 +106,7 @@ struct rtcc_ctx {
   BackboneParams* neck_p = nullptr;
   unsigned* neck_bar = nullptr;       // [kBarWords], zero between launches
   int* d_one = nullptr;               // [RTCC_MAX_AGENTS] = {1, 0, ...}: the head's one input
+  int* d_read = nullptr;              // [RTCC_MAX_AGENTS] presence flags of a read-back's fusion
   int post_kernels = 0;               // kernels of the post-join graph
   size_t img_elems = 0, feat_elems = 0;
   std::vector<ConvLayer> layers;      // the layer list (N tiles of a one-agent launch)
@@ -571,8 +572,7 @@ rtcc_status build_backbone(rtcc_ctx* c) {
     RS(dalloc(c, &c->neck_out, c->feat_elems * es));
     CK(cudaMemset(c->neck_out, 0, c->feat_elems * es));
   }
-  c->fused_neck = neck && (c->ms || g.fusion == RTCC_FUSE_MAX) &&
-                  !(g.flags & (RTCC_FLAG_KEEP_FUSED | RTCC_FLAG_LAYER_TIMES)) &&
+  c->fused_neck = neck && !(g.flags & (RTCC_FLAG_KEEP_FUSED | RTCC_FLAG_LAYER_TIMES)) &&
                   neck_head_ok(g.n_blocks, g.block_ch, g.up_stride, g.up_ch);
   const bool apart = c->ms || c->fused_neck;   // the deconvs are not layers of the branches
   for (int bi = 0; neck && bi < g.n_blocks; ++bi) {
@@ -785,26 +785,37 @@ rtcc_status capture_branch(rtcc_ctx* c, int k) {
   return capture_branch_graph(c, k, ph, false, &b.pill_host);
 }
 
+// Attention over the agents' feature slots, into the context's fused map; with
+// the same bytes as the kernel that runs the neck itself where that kernel
+// takes the network.
+FuseBlocksArgs slot_attention(rtcc_ctx* c, const int* present) {
+  FuseBlocksArgs fb{};
+  fb.n = 1;
+  fb.src[0] = c->feat_all;
+  fb.cells[0] = c->Wf * c->Hf;
+  fb.ch[0] = c->Cf;
+  fb.astride[0] = (long long)c->feat_elems;
+  fb.dst[0] = c->fused;
+  fb.present = present;
+  fb.K = c->K;
+  fb.attention = 1;
+  const rtcc_model_config& g = c->cfg;
+  fb.slot_order = g.up_stride[0] != 0 && neck_head_ok(g.n_blocks, g.block_ch, g.up_stride, g.up_ch);
+  return fb;
+}
+
 rtcc_status capture_post(rtcc_ctx* c) {
   const bool tl = (c->cfg.flags & RTCC_FLAG_TIMELINE) != 0;
   // multi-scale placement: fuse each block's outputs, run the neck once on the
   // fused maps, then the head over that one map (the max "fusion" of a single
   // input is the identity, so the tensor-core head kernel serves as the head).
-  // Single-scale attention takes the same two steps on the 384-channel slots:
-  // the bandwidth-bound fusion writes the fused map, the tensor-core kernel
-  // runs the head over it.
+  // Single-scale attention over stored 384-channel slots (where the neck kernel
+  // does not run the whole of it) takes the same two steps: the bandwidth-bound
+  // fusion writes the fused map, the tensor-core kernel runs the head over it.
   const bool attn1 = !c->ms && c->cfg.fusion == RTCC_FUSE_ATTN && fuse_tc_chunk(c->Cf, 1) > 0 && c->fused;
   FuseBlocksArgs fb{};
   if (attn1) {
-    fb.n = 1;
-    fb.src[0] = c->feat_all;
-    fb.cells[0] = c->Wf * c->Hf;
-    fb.ch[0] = c->Cf;
-    fb.astride[0] = (long long)c->feat_elems;
-    fb.dst[0] = c->fused;
-    fb.present = c->d_present;
-    fb.K = c->K;
-    fb.attention = 1;
+    fb = slot_attention(c, c->d_present);
     fb.span = c->fuse_span;
   } else if (c->ms) {
     fb.n = c->cfg.n_blocks;
@@ -838,6 +849,7 @@ rtcc_status capture_post(rtcc_ctx* c) {
     a.feat_h = c->Hf;
     a.present = c->ms ? c->d_one : c->d_present;
     a.K = c->ms ? 1 : c->K;
+    a.attention = !c->ms && c->cfg.fusion == RTCC_FUSE_ATTN;
     a.head_b = c->head_b;
     a.head_out = c->head_out;
     a.keys = c->keys;
@@ -849,7 +861,7 @@ rtcc_status capture_post(rtcc_ctx* c) {
     a.wait_budget = c->wait_budget;
     CK(neck_head_fill(a, c->bf16, &nh));
   }
-  const bool two_step = c->ms || attn1;
+  const bool two_step = c->ms || (attn1 && !c->fused_neck);
   const int K_head = two_step ? 1 : c->K;
   FuseArgs fa{};
   fa.feats = c->d_feat_ptrs;
@@ -939,12 +951,12 @@ rtcc_status capture_post(rtcc_ctx* c) {
     if (e == cudaSuccess && tl) e = record_node(c->ev_fuse1, c->post);
     if (e == cudaSuccess && c->ms && !c->fused_neck) e = launch_backbone(*c->neck_p, c->bf16, c->post);
     if (e == cudaSuccess)
-      e = c->fused_neck ? launch_neck_max_head(nh, c->bf16, c->post)
+      e = c->fused_neck ? launch_neck_head(nh, c->bf16, c->post)
                         : launch_fuse_max_head(tp, c->bf16, c->post);
   } else {
     if (e == cudaSuccess) {
       if (c->fused_neck)
-        e = launch_neck_max_head(nh, c->bf16, c->post);
+        e = launch_neck_head(nh, c->bf16, c->post);
       else if (use_tc)
         e = launch_fuse_max_head(tp, c->bf16, c->post);
       else
@@ -1058,6 +1070,7 @@ rtcc_status init_impl(rtcc_ctx* c, const float* weights) {
   {
     int one[RTCC_MAX_AGENTS] = {1};
     RS(dalloc(c, &c->d_one, sizeof(one)));
+    RS(dalloc(c, &c->d_read, sizeof(one)));
     CK(cudaMemcpy(c->d_one, one, sizeof(one), cudaMemcpyHostToDevice));
   }
   const size_t nkeys = decode_key_capacity(cells_f * g.anchors);
@@ -1820,7 +1833,21 @@ rtcc_status rtcc_get_tensor(rtcc_ctx* c, int32_t agent, int32_t which, uint16_t*
     CK(cudaStreamSynchronize(c->post));
     src = f;
     n = (size_t)c->Wf * c->Hf * c->Cf;
-    if (host_out && cap >= n && c->fused_neck) RS(run_neck(c, 0));
+    if (host_out && cap >= n && c->fused_neck) {
+      if (c->ms) {
+        RS(run_neck(c, 0));
+      } else {
+        // single-scale attention: the present agents' maps, then their fusion
+        int pres[RTCC_MAX_AGENTS] = {};
+        for (int k = 0; k < c->K; ++k) {
+          pres[k] = c->ctrl.present(k) ? 1 : 0;
+          if (pres[k]) RS(run_neck(c, k));
+        }
+        CK(cudaMemcpy(c->d_read, pres, sizeof(pres), cudaMemcpyHostToDevice));
+        CK(launch_fuse_blocks(slot_attention(c, c->d_read), c->bf16, c->post));
+        CK(cudaStreamSynchronize(c->post));
+      }
+    }
   } else if (which >= 10 && which < 10 + c->cfg.n_blocks) {
     if (!c->ms) return RTCC_E_STATE;
     CK(cudaStreamSynchronize(c->post));

@@ -206,6 +206,100 @@ __global__ void __launch_bounds__(kThreads, (ATTN || WIDE) ? 3 : 5) k_fuse_block
   }
 }
 
+// Attention over feature slots of C = 128 nb channels with every sum in the
+// order of the kernel that fuses without stored slots (k_neck_head), so that
+// both give the same bytes: the dot product as one chain over each 32
+// channels, those of the same 32 columns added over the nb blocks, then over
+// the four column groups; the softmax over all scores, the weights normalised
+// before the sums.  Half a warp per cell, 4 nb of its lanes own 32 channels
+// each; the maps are read twice.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 3) k_fuse_slots(const __grid_constant__ FuseBlocksArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  span_begin(a.span);
+  unsigned pres = 0;
+  for (int k = 0; k < a.K; ++k) pres |= (a.present[k] ? 1u : 0u) << k;
+  const int lane = threadIdx.x & 31, h0 = lane & 16, hl = lane & 15;
+  const int C = a.ch[0], nb = C / 128;
+  const bool mine = hl < 4 * nb;
+  const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < a.tasks[0]; w += warps) {
+    const int cell = (int)(2 * w) + (lane >> 4);
+    const bool valid = cell < a.cells[0];
+    const size_t off = (size_t)(valid ? cell : a.cells[0] - 1) * C + (size_t)(mine ? hl : 0) * 32;
+    const T* src = static_cast<const T*>(a.src[0]) + off;
+    auto load = [&](int k, uint32_t (&x)[16]) {
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const uint4 r = ld16(src + (size_t)k * a.astride[0] + 8 * v);
+        x[4 * v] = r.x;
+        x[4 * v + 1] = r.y;
+        x[4 * v + 2] = r.z;
+        x[4 * v + 3] = r.w;
+      }
+    };
+    uint32_t q[16];
+    load(0, q);
+    float s[RTCC_MAX_AGENTS], m = -INFINITY, den = 0.f;
+#pragma unroll
+    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) {
+      if (!((pres >> k) & 1u)) continue;
+      uint32_t x[16];
+      load(k, x);
+      float d = 0.f;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float2 u = Store<T>::unpack2(q[i]), v = Store<T>::unpack2(x[i]);
+        d = fmaf(u.x, v.x, d);
+        d = fmaf(u.y, v.y, d);
+      }
+      float part[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        part[g] = __shfl_sync(kFull, d, h0 + g);
+        for (int b = 1; b < nb; ++b) part[g] += __shfl_sync(kFull, d, h0 + 4 * b + g);
+      }
+      s[k] = __fmul_rn(part[0] + part[1] + part[2] + part[3], a.inv_sqrt_c[0]);
+      m = fmaxf(m, s[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) {
+      if (!((pres >> k) & 1u)) continue;
+      s[k] = expf(s[k] - m);
+      den += s[k];
+    }
+    const float inv = 1.f / den;
+    float f[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) f[i] = 0.f;
+#pragma unroll
+    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) {
+      if (!((pres >> k) & 1u)) continue;
+      const float wk = __fmul_rn(s[k], inv);
+      uint32_t x[16];
+      load(k, x);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float2 v = Store<T>::unpack2(x[i]);
+        f[2 * i] = fmaf(wk, v.x, f[2 * i]);
+        f[2 * i + 1] = fmaf(wk, v.y, f[2 * i + 1]);
+      }
+    }
+    if (valid && mine) {
+      uint4* out = reinterpret_cast<uint4*>(static_cast<T*>(a.dst[0]) + off);
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        out[v] = make_uint4(Store<T>::pack2(f[8 * v], f[8 * v + 1]), Store<T>::pack2(f[8 * v + 2], f[8 * v + 3]),
+                            Store<T>::pack2(f[8 * v + 4], f[8 * v + 5]), Store<T>::pack2(f[8 * v + 6], f[8 * v + 7]));
+    }
+  }
+  if (a.span) {
+    __syncthreads();
+    span_end(a.span);
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_fuse_blocks(FuseBlocksArgs a, bool bf16, cudaStream_t st) {
@@ -213,6 +307,8 @@ cudaError_t launch_fuse_blocks(FuseBlocksArgs a, bool bf16, cudaStream_t st) {
   long long work = 0;
   const bool wide = a.ch[0] == 384;
   if (wide && a.n != 1) return cudaErrorInvalidValue;
+  if (a.slot_order && (a.n != 1 || !a.attention || a.ch[0] < 128 || a.ch[0] > 384 || a.ch[0] % 128))
+    return cudaErrorInvalidValue;
   for (int b = 0; b < a.n; ++b) {
     if (!wide && a.ch[b] != 32 && a.ch[b] != 64 && a.ch[b] != 128 && a.ch[b] != 256)
       return cudaErrorInvalidValue;
@@ -222,7 +318,7 @@ cudaError_t launch_fuse_blocks(FuseBlocksArgs a, bool bf16, cudaStream_t st) {
     if ((reinterpret_cast<uintptr_t>(a.src[b]) | reinterpret_cast<uintptr_t>(a.dst[b])) & 15u ||
         (a.astride[b] * 2) % 16)
       return cudaErrorInvalidValue;
-    const int cpw = wide ? 2 : 32 / (a.ch[b] / 8);   // cells per warp task
+    const int cpw = wide || a.slot_order ? 2 : 32 / (a.ch[b] / 8);   // cells per warp task
     a.tasks[b] = (a.cells[b] + cpw - 1) / cpw;
     a.inv_sqrt_c[b] = 1.0f / sqrtf((float)a.ch[b]);
     work += a.tasks[b];
@@ -235,6 +331,9 @@ cudaError_t launch_fuse_blocks(FuseBlocksArgs a, bool bf16, cudaStream_t st) {
   if (blocks > 8LL * sms) blocks = 8LL * sms;       // grid-stride beyond 8 blocks per SM
   if (blocks < 1) blocks = 1;
   const dim3 g((unsigned)blocks), t(kThreads);
+  if (a.slot_order)
+    return bf16 ? launch_pdl(k_fuse_slots<__nv_bfloat16>, g, t, 0, st, a)
+                : launch_pdl(k_fuse_slots<__half>, g, t, 0, st, a);
   if (bf16) {
     if (wide)
       return a.attention ? launch_pdl(k_fuse_blocks<__nv_bfloat16, true, true>, g, t, 0, st, a)

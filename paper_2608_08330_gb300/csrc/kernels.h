@@ -283,6 +283,8 @@ struct FuseBlocksArgs {
   const int* present;                   // device [K] presence flags
   int K;
   int attention;                        // 0 = max, 1 = ego-query attention
+  int slot_order;                       // attention of one map of 128 to 384 channels with the
+                                        // sums in the order of neck_head.cu
   unsigned long long* span;             // device [3] kernel span stamps, or null
 };
 cudaError_t launch_fuse_blocks(FuseBlocksArgs a, bool bf16, cudaStream_t st);
@@ -311,7 +313,7 @@ int fuse_tc_chunk(int C, int K);
 int fuse_tc_stages(int C, int K);   // pipeline stages for that chunk
 cudaError_t launch_fuse_max_head(const FuseTcParams& p, bool bf16, cudaStream_t st);
 
-// Neck (deconvs of every block), max over the agents and head in one kernel
+// Neck (deconvs of every block), fusion over the agents and head in one kernel
 // (neck_head.cu), from the blocks' outputs.
 struct NeckHeadArgs {
   int n_blocks;
@@ -325,6 +327,7 @@ struct NeckHeadArgs {
   int feat_w, feat_h;                   // output map
   const int* present;                   // device [K]
   int K;
+  int attention;                        // 0: max, 1: ego-query attention (agent 0 present)
   const float* head_b;                  // device [16]
   float* head_out;                      // device [cells][16]
   uint32_t* keys;                       // device [cells][anchors] decode keys
@@ -345,6 +348,8 @@ struct NeckHeadParams {
   int Wf, Wq, Hq;                       // output row length; quotient grid (W' / S, H' / S)
   int tw, th, tiles_x, tiles;           // tiles of the quotient grid
   int K;
+  int attention;
+  float inv_sqrt_c;
   const int* present;
   const float* head_b;
   float* head_out;
@@ -361,7 +366,7 @@ struct NeckHeadParams {
 bool neck_head_ok(int n_blocks, const int* cin, const int* stride, int up_ch);
 void neck_head_tile(int W, int H, int* tw, int* th);
 cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P);
-cudaError_t launch_neck_max_head(const NeckHeadParams& p, bool bf16, cudaStream_t st);
+cudaError_t launch_neck_head(const NeckHeadParams& p, bool bf16, cudaStream_t st);
 
 // Dense 16-bit tensor map of any rank up to 5 (dims innermost first, strides
 // in bytes of dimensions 1 .. rank - 1).

@@ -1,9 +1,11 @@
-// The deconv neck, the cross-agent max and the 1x1 detection head in one
-// kernel (the shared post-join subgraph, Sec. III-B / Sec. IV-D, for the
-// element-wise max fusion), on the 5th-generation tensor cores.
+// The deconv neck, the cross-agent fusion and the 1x1 detection head in one
+// kernel (the shared post-join subgraph, Sec. III-B / Sec. IV-D), on the
+// 5th-generation tensor cores.
 //
 //   X_k[cell][128 b + c] = relu(bias_b[c] + sum_i W_b[sub][c][i] Y_kb[pixel][i])
-//   F[cell][.]           = max over present agents k of X_k[cell][.]
+//   F[cell][.]           = max over present agents k of X_k[cell][.], or
+//                          sum_k w_k X_k[cell][.], w = softmax over present k of
+//                          <X_0[cell], X_k[cell]> / sqrt(128 blocks)  (attention)
 //   out[cell][o]         = head_b[o] + sum_c W_head[o][c] F[cell][c],  o < 16
 //
 // with Y_kb agent k's output of backbone block b, pixel the input pixel under
@@ -20,6 +22,16 @@
 // The maximum is taken on the fp32 accumulators, before bias, ReLU and the
 // rounding to 16 bits: all three are monotone, so rounding the maximum gives
 // the very bits of the maximum of the rounded values.
+//
+// Attention needs the scores over all 384 channels before the first sum, so an
+// item makes two passes over blocks and agents: the first computes every X_k
+// (rounded to 16 bits, as stored maps are) and its dot product with the ego's,
+// the second computes it again and adds w_k X_k in fp32.  Computing twice costs
+// the MMAs of 21 GFLOP and the L2 reads of the blocks' outputs once more: 64 us
+// for 5 agents on the 352 x 100 map, near the 50 us of its 315 MB of L2 reads.
+// Storing the maps cost 68 us of deconvs in the branches' launch, 38 us of
+// fusion and 14 us of head.  Where the maps are stored all the same,
+// k_fuse_slots (fuse_blocks.cu) takes the sums in this kernel's order.
 //
 // Work item: 128 cells that share their position (sy, sx) modulo the largest
 // stride S, i.e. cells (S qy + sy, S qx + sx) of a tw x th rectangle of
@@ -39,11 +51,11 @@
 // operand of the head's N = 16 MMAs, which accumulate over the blocks in
 // channel order.
 //
-// Roles (800 threads): warps 0..15 max epilogue (tensor-memory lane quarter
-// warp % 4, columns 32 (warp / 4)), warps 16..19 head epilogue, warps 20..23
-// one TMA producer thread each (a thread's boxes complete one after another,
-// so the stages are dealt over four), warp 24 tensor-memory owner and MMA
-// issuer.  Every wait is bounded (an error bit, no hang); the summation order
+// Roles (800 threads; attention 768): warps 0..15 fusion epilogue
+// (tensor-memory lane quarter warp % 4, columns 32 (warp / 4)), warps 16..19
+// head epilogue, then four warps (attention three) with one TMA producer thread
+// each (a thread's boxes complete one after another, so the stages are dealt
+// over them), the last warp tensor-memory owner and MMA issuer.  Every wait is bounded (an error bit, no hang); the summation order
 // is fixed, so the output is bit-reproducible.
 #include <algorithm>
 #include <cmath>
@@ -59,10 +71,13 @@ namespace {
 constexpr int kEpiWarps = 16;
 constexpr int kHeadWarp0 = kEpiWarps;          // 4 head epilogue warps
 constexpr int kProdWarp0 = kHeadWarp0 + 4;
-constexpr int kProducers = 4;
-constexpr int kMmaWarp = kProdWarp0 + kProducers;
-constexpr int kThreads = (kMmaWarp + 1) * 32;
-constexpr int kStages = 4;                     // one per producer thread
+// Producer warps: attention has one less, which makes 24 warps and 80 registers
+// a thread instead of 72.  Its epilogue keeps its biases packed in shared memory
+// and loads 8 columns at a time for the same reason: with 50 words spilled the
+// kernel took 119 us instead of 64.
+constexpr int producers(bool attn) { return attn ? 3 : 4; }
+constexpr int threads(bool attn) { return (kProdWarp0 + producers(attn) + 1) * 32; }
+constexpr int kStages = 4;
 constexpr int kTile = 128;                     // cells per item (MMA M)
 constexpr int kUp = 128;                       // channels per deconv
 constexpr int kChunk = kTile * 64 * 2;         // 64 channels of 128 rows, 128-byte swizzle
@@ -78,7 +93,9 @@ constexpr int kHOff = kFOff + 2 * kChunk;
 constexpr int kBarOff = kHOff + RTCC_MAX_BLOCKS * 2 * kHeadChunk;
 constexpr int kSmem = kBarOff + 256 + 1024;    // barriers; alignment to 1024
 static_assert(kSmem <= 227 * 1024 - 2048, "shared memory budget (with the static arrays)");
-static_assert(kStages == kProducers, "stage s belongs to producer thread s");
+// the producers take turns on the stages: a thread's wait for a stage rules out
+// the phase before the one its next wait is for
+static_assert(producers(false) <= kStages, "phase parity");
 
 // tile t of a CTA's range: position (sy, sx), origin in the quotient grid
 struct NhItem {
@@ -96,8 +113,13 @@ __device__ __forceinline__ NhItem item_at(const NeckHeadParams& P, int t) {
   return I;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_constant__ NeckHeadParams P) {
+// barrier among the 16 epilogue warps (named barrier 1)
+__device__ __forceinline__ void epilogue_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory"); }
+
+// ATTN: attention fusion instead of the maximum (see the top of the file).
+template <typename T, bool ATTN>
+__global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_constant__ NeckHeadParams P) {
+  constexpr int kProducers = producers(ATTN), kMmaWarp = kProdWarp0 + kProducers, kThreads = threads(ATTN);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -119,6 +141,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
   __shared__ __align__(16) float s_bias[RTCC_MAX_BLOCKS][kUp];
   __shared__ int s_list[RTCC_MAX_AGENTS];
   __shared__ int s_kp;
+  __shared__ float s_w[ATTN ? RTCC_MAX_AGENTS : 1][ATTN ? kTile : 1];   // an item's weights, agents in list order
 
   const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
   const int lane = threadIdx.x & 31;
@@ -151,7 +174,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
-  for (int i = threadIdx.x; i < nb * kUp; i += kThreads) s_bias[i / kUp][i % kUp] = P.bias[i / kUp][i % kUp];
+  // the biases; for attention two a word in the storage type, which holds them
+  uint32_t* const bias2 = reinterpret_cast<uint32_t*>(&s_bias[0][0]);
+  if (ATTN) {
+    for (int i = threadIdx.x; i < nb * kUp / 2; i += kThreads) {
+      const float* b = P.bias[i / (kUp / 2)] + i % (kUp / 2) * 2;
+      bias2[i] = Store<T>::pack2(b[0], b[1]);
+    }
+  } else {
+    for (int i = threadIdx.x; i < nb * kUp; i += kThreads) s_bias[i / kUp][i % kUp] = P.bias[i / kUp][i % kUp];
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -196,7 +228,134 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
   __syncthreads();
   const int Kp = s_kp;
 
-  if (warp < kEpiWarps) {
+  constexpr int kPasses = ATTN ? 2 : 1;        // passes over the agents per item
+  if (warp < kEpiWarps && ATTN) {
+    // ---------------- attention: scores, softmax, weighted sums ----------------
+    const int qd = warp & 3, cg = warp >> 2;
+    const int row = qd * 32 + lane;
+    const uint32_t tcol = tmem + (static_cast<uint32_t>(qd * 32) << 16) + (uint32_t)(cg * 32);
+    uint8_t* frow = fsm + (cg >> 1) * kChunk + row * 128;
+    float* part = reinterpret_cast<float*>(fsm);   // [agent][column group][row] score parts
+    uint32_t st = 0, ph = 0;
+    bool alive = true;
+    // 8 columns from column 8 h on of the step in hand, rounded after bias and
+    // ReLU, two a word (8 at a time, to stay within a thread's registers)
+    auto rounded8 = [&](int h, const uint32_t* bias, uint32_t (&x)[4]) {
+      uint32_t r[8];
+      tmem_ld8_issue(tcol + (st % kAccs) * kUp + 8 * h, r);
+      const uint4 pb = *reinterpret_cast<const uint4*>(bias + 4 * h);
+      const uint32_t bb[4] = {pb.x, pb.y, pb.z, pb.w};
+      tmem_ld_wait();
+      tmem_reg_fence(r);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 b = Store<T>::unpack2(bb[i]);
+        x[i] = Store<T>::relu2(Store<T>::pack2(__uint_as_float(r[2 * i]) + b.x, __uint_as_float(r[2 * i + 1]) + b.y));
+      }
+    };
+    auto wait_full = [&]() {
+      if (alive && !mbar_wait(&accfull[st % kAccs], (st / kAccs) & 1, P.wait_budget)) {
+        if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
+        alive = false;
+      }
+      tc_fence_after();
+    };
+    auto release = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&accempty[st % kAccs]);
+    };
+    auto wait_fempty = [&]() {                 // the head MMAs of the block before have read the fused chunk
+      if (alive && !mbar_wait(fempty, (ph & 1) ^ 1, P.wait_budget)) {
+        if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
+        alive = false;
+      }
+    };
+    for (int t = lo; t < hi; ++t) {
+      // First pass: <X_ego, X_k> over this thread's channels of every block, in
+      // the fused chunk's memory, which is idle until the second pass.
+      wait_fempty();
+      float* mine = part + cg * kTile + row;   // agent k's part: + 4 k kTile
+      for (int b = 0; b < nb; ++b) {
+        const uint32_t* bias = bias2 + b * (kUp / 2) + cg * 16;   // of this thread's 32 channels
+        uint32_t ego[16];
+        for (int k = 0; k < Kp; ++k, ++st) {
+          wait_full();
+          float d = 0.f;
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            uint32_t x[4];
+            rounded8(h, bias, x);
+            if (h == 3) release();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              if (k == 0) ego[4 * h + i] = x[i];
+              const float2 a = Store<T>::unpack2(ego[4 * h + i]), c = Store<T>::unpack2(x[i]);
+              d = fmaf(a.x, c.x, d);
+              d = fmaf(a.y, c.y, d);
+            }
+          }
+          mine[4 * k * kTile] = b == 0 ? d : mine[4 * k * kTile] + d;
+        }
+      }
+      epilogue_sync();
+      // the column groups' parts meet: group 0 takes the softmax, a row a thread
+      if (cg == 0) {
+        float w[RTCC_MAX_AGENTS], m = -INFINITY, den = 0.f;
+#pragma unroll
+        for (int j = 0; j < RTCC_MAX_AGENTS; ++j) {
+          if (j < Kp) {
+            const float* q = part + j * 4 * kTile + row;
+            w[j] = __fmul_rn(q[0] + q[kTile] + q[2 * kTile] + q[3 * kTile], P.inv_sqrt_c);
+            m = fmaxf(m, w[j]);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < RTCC_MAX_AGENTS; ++j) {
+          w[j] = j < Kp ? expf(w[j] - m) : 0.f;
+          den += w[j];
+        }
+        const float inv = 1.f / den;
+#pragma unroll
+        for (int j = 0; j < RTCC_MAX_AGENTS; ++j) s_w[j][row] = __fmul_rn(w[j], inv);
+      }
+      epilogue_sync();                         // the parts have been read, the weights written
+      // second pass: the weighted sums
+      for (int b = 0; b < nb; ++b, ++ph) {
+        const uint32_t* bias = bias2 + b * (kUp / 2) + cg * 16;
+        float f[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) f[i] = 0.f;
+        for (int k = 0; k < Kp; ++k, ++st) {
+          const float wk = s_w[k][row];
+          wait_full();
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            uint32_t x[4];
+            rounded8(h, bias, x);
+            if (h == 3) release();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float2 c = Store<T>::unpack2(x[i]);
+              f[8 * h + 2 * i] = fmaf(wk, c.x, f[8 * h + 2 * i]);
+              f[8 * h + 2 * i + 1] = fmaf(wk, c.y, f[8 * h + 2 * i + 1]);
+            }
+          }
+        }
+        wait_fempty();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float* v = f + 8 * j;
+          *reinterpret_cast<uint4*>(frow + ((((cg & 1) * 4 + j) ^ (row & 7)) << 4)) =
+              make_uint4(Store<T>::pack2(v[0], v[1]), Store<T>::pack2(v[2], v[3]), Store<T>::pack2(v[4], v[5]),
+                         Store<T>::pack2(v[6], v[7]));
+        }
+        fence_async_smem();                    // generic writes -> the MMA
+        __syncwarp();
+        if (lane == 0) mbar_arrive(fready);
+      }
+    }
+  } else if (warp < kEpiWarps) {
     // ---------------- running max, bias + ReLU + rounding ----------------
     const int qd = warp & 3, cg = warp >> 2;
     const int row = qd * 32 + lane;
@@ -301,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
     // ---------------- TMA producers (one thread in each of 4 warps) ----------------
     if (lane == 0 && lo < hi) {
       const uint32_t bytes = (uint32_t)(P.tw * P.th * 128);
-      uint32_t it = 0, loads = 1, mine = 0;    // weight loads so far; A boxes of this thread
+      uint32_t it = 0, loads = 1, mine = 0;    // weight loads so far; this thread's last stage + 1
       int cur = item_at(P, lo).sub;
       bool alive = true;
       for (int t = lo; t < hi && alive; ++t) {
@@ -316,21 +475,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
           ++loads;
           cur = I.sub;
         }
-        for (int b = 0; b < nb && alive; ++b) {
+        for (int pb = 0; pb < kPasses * nb && alive; ++pb) {
+          const int b = pb < nb ? pb : pb - nb;
           const int ox = I.sx / P.s[b], oy = I.sy / P.s[b];
           const int nc = P.cin[b] / 64;
           for (int k = 0; k < Kp && alive; ++k) {
             const int agent = s_list[k];
             for (int c = 0; c < nc; ++c, ++it) {
               if ((int)(it % kProducers) != pid) continue;
-              if (!mbar_wait(&empty[pid], ((it / kStages) & 1) ^ 1, P.wait_budget)) {
+              const uint32_t s = it % kStages;
+              if (!mbar_wait(&empty[s], ((it / kStages) & 1) ^ 1, P.wait_budget)) {
                 alive = false;
                 break;
               }
-              mbar_arrive_expect_tx(&full[pid], bytes);
-              tma_load_5d(smem + pid * kChunk, &P.in[b], &full[pid], ox * P.cin[b] + c * 64, I.x0, oy, I.y0,
-                          agent);
-              ++mine;
+              mbar_arrive_expect_tx(&full[s], bytes);
+              tma_load_5d(smem + s * kChunk, &P.in[b], &full[s], ox * P.cin[b] + c * 64, I.x0, oy, I.y0, agent);
+              mine = it + 1;
             }
           }
         }
@@ -338,7 +498,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
       if (!alive) {
         atomicOr(P.err, ERR_WAIT_FUSE);
         // this thread's last box may still be in flight into the CTA's memory
-        if (mine > 0) (void)mbar_wait(&full[pid], (mine - 1) & 1, P.wait_budget);
+        if (mine > 0)
+          (void)mbar_wait(&full[(mine - 1) % kStages], ((mine - 1) / kStages) & 1, P.wait_budget);
         (void)mbar_wait(wfull, (loads - 1) & 1, P.wait_budget);
       }
     }
@@ -391,8 +552,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
         ++loads;
         cur = sub;
       }
-      uint32_t w_lo = lo0 + (kWOff >> 4);      // block b's first weight chunk
-      for (int b = 0; b < nb && alive; ++b) {
+      uint32_t w_lo = 0;                       // block b's first weight chunk
+      for (int ps = 0; ps < kPasses * nb && alive; ++ps) {
+        const int b = ps < nb ? ps : ps - nb;
+        const bool head = ps >= (kPasses - 1) * nb;   // the pass whose sums the head reads
+        if (b == 0) w_lo = lo0 + (kWOff >> 4);
         const int nc = P.cin[b] / 64;
         for (int k = 0; k < Kp && alive; ++k, ++st) {
           const uint32_t buf = st % kAccs;
@@ -414,10 +578,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_neck_max_head(const __grid_cons
           if (pend && alive) flush();
         }
         if (pend && alive) flush();            // no agent present
-        pend = true;
-        pb = b;
-        pn = t - lo;
-        pph = ph++;
+        if (head) {
+          pend = true;
+          pb = b;
+          pn = t - lo;
+          pph = ph++;
+        }
         w_lo += nc * (kChunk >> 4);
       }
     }
@@ -499,6 +665,8 @@ cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P) 
       tmap_2d(&P->wh, a.head_w, bf16, (uint64_t)(a.n_blocks * kUp), kFuseHeadOut, 64, kFuseHeadOut, 128);
   if (e != cudaSuccess) return e;
   P->K = a.K;
+  P->attention = a.attention;
+  P->inv_sqrt_c = 1.0f / sqrtf((float)(a.n_blocks * kUp));
   P->present = a.present;
   P->head_b = a.head_b;
   P->head_out = a.head_out;
@@ -512,7 +680,7 @@ cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P) 
   return cudaSuccess;
 }
 
-cudaError_t launch_neck_max_head(const NeckHeadParams& p, bool bf16, cudaStream_t st) {
+cudaError_t launch_neck_head(const NeckHeadParams& p, bool bf16, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -522,10 +690,11 @@ cudaError_t launch_neck_max_head(const NeckHeadParams& p, bool bf16, cudaStream_
   if (items < 1 || sms < 1) return cudaErrorInvalidValue;
   const int rounds = (items + sms - 1) / sms;
   const int grid = (items + rounds - 1) / rounds;
-  auto kern = bf16 ? k_neck_max_head<__nv_bfloat16> : k_neck_max_head<__half>;
+  auto kern = p.attention ? (bf16 ? k_neck_head<__nv_bfloat16, true> : k_neck_head<__half, true>)
+                          : (bf16 ? k_neck_head<__nv_bfloat16, false> : k_neck_head<__half, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(grid), dim3(kThreads), kSmem, st, p);
+  return launch_pdl(kern, dim3(grid), dim3(threads(p.attention != 0)), kSmem, st, p);
 }
 
 }  // namespace rtcc

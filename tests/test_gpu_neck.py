@@ -1,8 +1,8 @@
-"""The post-join kernel that runs the deconv neck, the max over the agents and
+"""The post-join kernel that runs the deconv neck, the fusion over the agents and
 the head from the blocks' outputs, against the path that stores the neck's maps
-(RTCC_FLAG_KEEP_FUSED): the same sums, so the same bytes, for tiles that are
-ragged, single and narrow, one to three blocks, absent agents and both storage
-types; and the feature maps, which are then computed when they are read."""
+(RTCC_FLAG_KEEP_FUSED), for tiles that are ragged, single and narrow, one to
+three blocks, absent agents and both storage types: the same sums, so the same
+bytes; and the feature maps, which are then computed when they are read."""
 import dataclasses
 
 import pytest
@@ -55,6 +55,37 @@ def test_neck_max_head_matches_the_stored_maps(R, cfg, absent):
                         [R.rtcc_get_tensor(ctx, k, R.TENSOR_FEAT) for k in range(cfg.n_agents) if k not in absent])
                 got.append((R.rtcc_get_head(ctx, cfg.feat_h, cfg.feat_w).tobytes(), boxes.tobytes(),
                             [m.tobytes() for m in maps]))
+        finally:
+            R.rtcc_destroy(ctx)
+    assert all(g == got[0] for g in got[1:])
+
+
+ATTN = [
+    ("one tile of one pixel, the ego alone", _cfg(8, 8, 1, fusion="attn"), ()),
+    ("one narrow column", _cfg(8, 1040, 2, "bf16", fusion="attn"), ()),
+    ("ragged, several positions a CTA", _cfg(328, 184, 3, "bf16", fusion="attn"), (1,)),
+    ("all agents, 25 rows", _cfg(704, 200, 8, fusion="attn"), ()),
+    ("all but the ego and one absent", _cfg(72, 40, 8, fusion="attn"), (1, 2, 3, 4, 6, 7)),
+    ("one block", _cfg(40, 24, 3, blocks=((2, 128, 2),), ups=(1,), fusion="attn"), ()),
+    ("two blocks, strides 2 and 4", _cfg(48, 40, 2, "bf16", blocks=((1, 64, 1), (1, 256, 2)), ups=(1, 2),
+                                         fusion="attn"), ()),
+]
+
+
+@pytest.mark.parametrize("cfg,absent", [c[1:] for c in ATTN], ids=[c[0] for c in ATTN])
+def test_neck_attention_head_matches_the_stored_maps(R, cfg, absent):
+    # the path that stores the maps takes its sums in the same order
+    pts = [synth.points_for(cfg, 0, k) for k in range(cfg.n_agents)]
+    got = []
+    for f in (0, R.FLAG_KEEP_FUSED):
+        ctx, w = U.make_ctx(cfg, flags=f)
+        try:
+            for mode in (R.MODE_RTCC, R.MODE_BARRIER):
+                boxes = U.run_frame(ctx, cfg, pts, list(range(cfg.n_agents)), mode, absent=absent)
+                got.append((R.rtcc_get_head(ctx, cfg.feat_h, cfg.feat_w).tobytes(), boxes.tobytes(),
+                            R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes(),
+                            [R.rtcc_get_tensor(ctx, k, R.TENSOR_FEAT).tobytes()
+                             for k in range(cfg.n_agents) if k not in absent]))
         finally:
             R.rtcc_destroy(ctx)
     assert all(g == got[0] for g in got[1:])
