@@ -42,6 +42,7 @@ namespace {
 
 constexpr int kNmsThreads = 256;
 constexpr int kNmsWarps = kNmsThreads / 32;
+constexpr int kNmsBlocksPerSm = 2;
 constexpr int kNmsWords = kDecodeKeep / 32;     // mask words per row at most
 
 // One box: centre, heading (cos, sin) and half extents.
@@ -324,10 +325,12 @@ cudaError_t launch_nms(const NmsArgs& a, cudaStream_t st) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  // enough warps for the pair tests of a full list, at most one block per SM
+  // enough warps for the pair tests of a full list, up to kNmsBlocksPerSm
+  // blocks per SM (512 boxes: 4352 tests of a row against 32 boxes, which one
+  // block per SM takes in four rounds)
   const int tasks = a.max_boxes * ((a.max_boxes + 31) / 32);
   int grid = (tasks + kNmsWarps - 1) / kNmsWarps;
-  if (grid > sms) grid = sms;
+  if (grid > kNmsBlocksPerSm * sms) grid = kNmsBlocksPerSm * sms;
   if (grid < 1) grid = 1;
   DetResultHeader* hdr = static_cast<DetResultHeader*>(a.out);
   rtcc_box* boxes = reinterpret_cast<rtcc_box*>(hdr + 1);
@@ -348,19 +351,19 @@ namespace {
 // go out of and the kept ones come back into, their device copy with the
 // kernel's scratch, and a stream.  Allocating these per call (cudaMalloc,
 // stream creation, cudaFree with its device-wide synchronisation) and reading
-// the result back with two synchronous copies took most of a call: 210 us for
-// 128 boxes and 231 for 512, against 39 and 54 with a kept workspace and the
-// kernel's own stores into the pinned block.
+// the result back with two synchronous copies took most of a call: 217 us for
+// 128 boxes and 243 for 512, against 35 and 45 with a kept workspace, one copy
+// in and the kernel's own stores into the pinned block.
 struct NmsSpace {
   static constexpr size_t kBoxes = sizeof(rtcc_box) * kDecodeKeep;
-  // device copy / pinned source: the boxes, then {count, error word}
-  static constexpr size_t kCount = (kBoxes + 15) / 16 * 16;
-  static constexpr size_t kIn = kCount + 16;
-  static constexpr size_t kTicket = kIn;                      // device only
+  // device copy / pinned source: {count, error word}, then the boxes, so that
+  // what a call uses is one copy
+  static constexpr size_t kIn = 16;
+  static constexpr size_t kTicket = (kIn + kBoxes + 15) / 16 * 16;   // device only
   static constexpr size_t kMask = kTicket + 16;
   static constexpr size_t kMaskBytes = sizeof(uint32_t) * kDecodeKeep * kNmsWords;
   // pinned only: the done word, then the result block
-  static constexpr size_t kDone = kIn;
+  static constexpr size_t kDone = kTicket;
   static constexpr size_t kRes = kDone + 16;
   static constexpr size_t kHost = kRes + sizeof(DetResultHeader) + kBoxes;
 
@@ -468,21 +471,17 @@ NmsPool& nms_pool() {
 // The kernel on n boxes with workspace s; false on a CUDA error.
 bool nms_on(NmsSpace& s, const rtcc_box* host_in, int n, float iou, rtcc_box* host_out, int* n_out) {
   const size_t in_b = (size_t)n * sizeof(rtcc_box);
-  if (n > 0) std::memcpy(s.host, host_in, in_b);
-  int* cnt = reinterpret_cast<int*>(s.host + NmsSpace::kCount);
+  if (n > 0) std::memcpy(s.host + NmsSpace::kIn, host_in, in_b);
+  int* cnt = reinterpret_cast<int*>(s.host);
   cnt[0] = n;
   cnt[1] = 0;
   volatile int* done = reinterpret_cast<volatile int*>(s.host + NmsSpace::kDone);
   *done = 0;
   std::atomic_thread_fence(std::memory_order_seq_cst);
-  // the boxes in use, then the count and the error word
-  if (n > 0 && cudaMemcpyAsync(s.dev, s.host, in_b, cudaMemcpyHostToDevice, s.st) != cudaSuccess) return false;
-  if (cudaMemcpyAsync(s.dev + NmsSpace::kCount, s.host + NmsSpace::kCount, 16, cudaMemcpyHostToDevice, s.st) !=
-      cudaSuccess)
-    return false;
-  int* words = reinterpret_cast<int*>(s.dev + NmsSpace::kCount);
+  if (cudaMemcpyAsync(s.dev, s.host, NmsSpace::kIn + in_b, cudaMemcpyHostToDevice, s.st) != cudaSuccess) return false;
+  int* words = reinterpret_cast<int*>(s.dev);
   NmsArgs a{};
-  a.in = reinterpret_cast<const rtcc_box*>(s.dev);
+  a.in = reinterpret_cast<const rtcc_box*>(s.dev + NmsSpace::kIn);
   a.n_in = words;
   a.ticket = reinterpret_cast<unsigned*>(s.dev + NmsSpace::kTicket);
   a.err = words + 1;
