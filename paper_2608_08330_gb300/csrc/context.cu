@@ -156,6 +156,7 @@ struct rtcc_ctx {
   cudaEvent_t ev_post0 = nullptr, ev_fuse0 = nullptr, ev_fuse1 = nullptr, ev_post1 = nullptr;
   // frame bookkeeping
   bool post_launched = false;
+  int post_present[RTCC_MAX_AGENTS] = {};   // the agents of the last post-join
   bool closed_pending = false;
   double t_last_event = 0.0;
   rtcc_frame_info info{};
@@ -1277,8 +1278,10 @@ rtcc_status launch_batch(rtcc_ctx* c) {
 rtcc_status launch_post(rtcc_ctx* c) {
   // the presence flags are set on the device by the branches that ran (their
   // first kernel) and cleared by the decode kernel
-  for (int k = 0; k < c->K; ++k)
-    if (c->ctrl.present(k)) CK(cudaStreamWaitEvent(c->post, c->br[k].feat_ev, 0));
+  for (int k = 0; k < c->K; ++k) {
+    c->post_present[k] = c->ctrl.present(k) ? 1 : 0;
+    if (c->post_present[k]) CK(cudaStreamWaitEvent(c->post, c->br[k].feat_ev, 0));
+  }
   *c->h_done = 0;                                 // the decode kernel sets it when the boxes are written
   std::atomic_thread_fence(std::memory_order_seq_cst);
   CK(cudaGraphLaunch(c->post_exec, c->post));
@@ -1837,13 +1840,11 @@ rtcc_status rtcc_get_tensor(rtcc_ctx* c, int32_t agent, int32_t which, uint16_t*
       if (c->ms) {
         RS(run_neck(c, 0));
       } else {
-        // single-scale attention: the present agents' maps, then their fusion
-        int pres[RTCC_MAX_AGENTS] = {};
-        for (int k = 0; k < c->K; ++k) {
-          pres[k] = c->ctrl.present(k) ? 1 : 0;
-          if (pres[k]) RS(run_neck(c, k));
-        }
-        CK(cudaMemcpy(c->d_read, pres, sizeof(pres), cudaMemcpyHostToDevice));
+        // single-scale attention: the maps of the last post-join's agents (a
+        // new frame may have begun), then their fusion
+        for (int k = 0; k < c->K; ++k)
+          if (c->post_present[k]) RS(run_neck(c, k));
+        CK(cudaMemcpy(c->d_read, c->post_present, sizeof(c->post_present), cudaMemcpyHostToDevice));
         CK(launch_fuse_blocks(slot_attention(c, c->d_read), c->bf16, c->post));
         CK(cudaStreamSynchronize(c->post));
       }

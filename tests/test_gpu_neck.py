@@ -86,6 +86,9 @@ def test_neck_attention_head_matches_the_stored_maps(R, cfg, absent):
                             R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes(),
                             [R.rtcc_get_tensor(ctx, k, R.TENSOR_FEAT).tobytes()
                              for k in range(cfg.n_agents) if k not in absent]))
+            # the last frame's fused map, also once the next frame has begun
+            assert R.rtcc_frame_begin(ctx, 9, 0.0) == R.OK
+            assert R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes() == got[-1][2]
         finally:
             R.rtcc_destroy(ctx)
     assert all(g == got[0] for g in got[1:])
