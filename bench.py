@@ -54,7 +54,7 @@ METRIC = "complete-detection latency p50/p99 ms RTCC vs barrier; conv TFLOP/s, f
 # dram__bytes_read.sum + dram__bytes_write.sum per k_backbone launch from an
 # ncu capture of this build, keyed by the launch's agent count; None until
 # captured (and again once the kernel changes)
-BACKBONE_TRAFFIC = {8: 542_687_232, 1: 28_923_392}   # profiles/backbone_stress8.md
+BACKBONE_TRAFFIC = {8: 274_263_296, 1: 25_010_944}   # profiles/backbone_neck_704x200.md
 WORKLOAD = "stress8"
 DATA = ("synthetic: seeded uniform + Gaussian-cluster point clouds, He-normal fp32 weights "
         "rounded to fp16, seeded arrival traces (OPV2V and the trained OpenCOOD model are not "
@@ -77,8 +77,9 @@ def _peaks():
 
 
 def conv_flops(cfg) -> float:
-    """Algorithmic FLOPs of one encoder branch's convs and deconvs (2 per MAC)."""
-    return sum(fl for _, fl in layer_table(cfg))
+    """Algorithmic FLOPs of one branch's convs (2 per MAC), which the backbone
+    launch runs; the neck's deconvs are part of the post-join kernel."""
+    return sum(fl for name, fl in layer_table(cfg) if "deconv" not in name)
 
 
 def layer_table(cfg):
@@ -102,10 +103,15 @@ def layer_table(cfg):
 
 
 def fusion_bytes(cfg, k_present: int) -> float:
-    """Algorithmic bytes of the fusion+head kernel: each present slot read
-    once (16-bit), the fp32 head map written once."""
-    cells = cfg.feat_w * cfg.feat_h
-    return float(k_present * cells * cfg.feat_ch * 2 + cells * 16 * 4)
+    """Algorithmic bytes of the neck + fusion + head kernel: the present agents'
+    block outputs and the deconv weights read once (16-bit), the fp32 head map
+    written once."""
+    w, h, per_agent, weights = cfg.grid_w, cfg.grid_h, 0, 0
+    for (_, ch, st), s in zip(cfg.blocks, cfg.up_strides):
+        w, h = w // st, h // st
+        per_agent += w * h * ch * 2
+        weights += s * s * cfg.up_ch * ch * 2
+    return float(k_present * per_agent + weights + cfg.feat_w * cfg.feat_h * 16 * 4)
 
 
 def pfn_bytes(cfg, n_pillars: int, n_kept: int, n_raw: int) -> float:
@@ -752,8 +758,8 @@ def run_ours(args):
                    "inputs": "value: payloads resident in HBM before release; e2e: payloads in "
                              "pinned host memory, read on release inside the measured span",
                    "replicas": world},
-        "roofline": {"kernel": "k_backbone (persistent tcgen05 implicit-GEMM backbone: 13 convs + "
-                               "3 deconvs of every agent in the launch)",
+        "roofline": {"kernel": "k_backbone (persistent tcgen05 implicit-GEMM backbone: the 13 convs "
+                               "of every agent in the launch)",
                      "bound": "tensor", "achieved": sig(enc_tflops), "peak": tflops_peak,
                      "unit": "TFLOP/s",
                      "frac": sig(enc_tflops / tflops_peak, 3) if enc_tflops else None,
