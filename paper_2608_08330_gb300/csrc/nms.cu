@@ -42,7 +42,7 @@ namespace {
 
 constexpr int kNmsThreads = 256;
 constexpr int kNmsWarps = kNmsThreads / 32;
-constexpr int kNmsBlocksPerSm = 2;
+constexpr int kNmsBlocksPerSm = 4;
 constexpr int kNmsWords = kDecodeKeep / 32;     // mask words per row at most
 
 // One box: centre, heading (cos, sin) and half extents.
@@ -325,10 +325,14 @@ cudaError_t launch_nms(const NmsArgs& a, cudaStream_t st) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  // enough warps for the pair tests of a full list, up to kNmsBlocksPerSm
-  // blocks per SM (512 boxes: 4352 tests of a row against 32 boxes, which one
-  // block per SM takes in four rounds)
-  const int tasks = a.max_boxes * ((a.max_boxes + 31) / 32);
+  // one warp for each pair-test task of a full list (the kernel's own count),
+  // up to kNmsBlocksPerSm blocks per SM, which all 4352 tasks of 512 boxes fit
+  // in: a call of 512 boxes takes 44 us, against 47 with two blocks per SM and
+  // two rounds.  (256 boxes: 144 blocks, where a grid for the full square of
+  // rows and words had 256; the time is the same.)
+  const int W = (a.max_boxes + 31) / 32;
+  int tasks = 0;
+  for (int c = 0; c < W; ++c) tasks += std::min(32, a.max_boxes - 32 * c) * (W - c);
   int grid = (tasks + kNmsWarps - 1) / kNmsWarps;
   if (grid > kNmsBlocksPerSm * sms) grid = kNmsBlocksPerSm * sms;
   if (grid < 1) grid = 1;
@@ -352,7 +356,7 @@ namespace {
 // kernel's scratch, and a stream.  Allocating these per call (cudaMalloc,
 // stream creation, cudaFree with its device-wide synchronisation) and reading
 // the result back with two synchronous copies took most of a call: 217 us for
-// 128 boxes and 243 for 512, against 35 and 45 with a kept workspace, one copy
+// 128 boxes and 243 for 512, against 35 and 44 with a kept workspace, one copy
 // in and the kernel's own stores into the pinned block.
 struct NmsSpace {
   static constexpr size_t kBoxes = sizeof(rtcc_box) * kDecodeKeep;

@@ -80,3 +80,15 @@ def test_nms_threads_and_shrinking_lists(R):
         for got in ex.map(turn, range(8)):
             for i, out in got:
                 assert out.tobytes() == want[i].tobytes()
+
+
+@pytest.mark.parametrize("n", [64, 65, 224, 255, 256, 257, 481, 512])
+def test_nms_suppressors_in_any_earlier_chunk(R, n):
+    """A row of boxes that overlap their neighbours, ranked at random: what
+    removes a box lies in its own 32-box chunk, the one before or any earlier
+    one, in odd and even numbers of chunks, the last one full or not."""
+    rng = np.random.default_rng(n)
+    x = rng.permutation(n) * 1.7
+    b = _boxes(np.column_stack([x, np.zeros(n), np.full(n, 4.0), np.full(n, 1.8), np.zeros(n)]))
+    kept = U.check_nms(b, R.rtcc_nms(b, 0.2), 0.2)
+    assert n // 4 <= len(kept) <= n // 2 + 1           # IoU 0.40 to a neighbour, 0.08 two on
