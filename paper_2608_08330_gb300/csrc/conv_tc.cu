@@ -523,11 +523,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
         // Every item of the same agent in the layer this one reads has been
         // stored: waited for once per agent, before the first box of its input
         // (with stamps every agent's, so that the layers' spans follow each
-        // other).
+        // other; a dsm layer too, whose exchange needs the receive buffers of
+        // the layers before it to have been read, see the epilogue).
         int ready = -1;                          // batch slot known to be ready
+        const bool all = P.stamps != nullptr || S.dsm != 0;
         auto input_ready = [&](int slot) -> bool {
           if (S.wait_layers == 0 || slot == ready) return true;
-          const int j0 = P.stamps ? 0 : slot, j1 = P.stamps ? P.n_batch : slot + 1;
+          const int j0 = all ? 0 : slot, j1 = all ? P.n_batch : slot + 1;
           for (int j = j0; j < j1; ++j) {
             if (!grid_wait(&P.grid_bar[(S.wait_layers - 1) * RTCC_MAX_AGENTS + j],
                            (unsigned)S.wait_items + stall, budget))
@@ -883,8 +885,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
           // its 64 partial columns into its own shared memory by owner; one
           // bulk copy per peer moves the peer's slot into the peer's receive
           // slot (counted on the peer's mbarrier); each owner sums the slices in
-          // slice order and stores its channels in 16-channel TMA boxes.  The
-          // slots are rewritten only after the next item's bulk_wait_read_all.
+          // slice order and stores its channels from registers, 16 at a time.
+          // The own slots are rewritten only after the next item's
+          // bulk_wait_read_all.
+          //
+          // The receive buffer and its barrier are one per CTA, and no peer is
+          // told when they are free: the order of the layers has to say so.
+          // This item's A operand was loaded behind the counters of every agent
+          // of the layer it reads (input_ready); each of those items had its
+          // agent's items of the layer before, and so on down, so every item of
+          // every earlier layer has been counted.  A CTA takes at most one item
+          // of a dsm layer and counts it after it has summed what it received:
+          // when a copy of this layer leaves, no receive buffer of an earlier
+          // one is still waited for or read, whichever agents the ranks had.
+          // (Waiting for the item's own agent only, as other layers do, a rank
+          // could send its next agent's slices into a buffer in use: `rot` gives
+          // a cluster different agents from layer to layer.)
           const int Sp = S.splits;
           const int CW = 64 / Sp, G16 = CW / 16;
           const int z = I.z;
