@@ -85,6 +85,8 @@ struct PillarBufs {
   int clear_all;         // 1: the pass clears all of image and cell2pillar (their
                          // content is unknown); 0: they hold the previous pass's
                          // output, and only its np_prev pillar cells are cleared
+  int caller_weights;    // 1: the weights are the caller's and may be written by the work
+                         // before the pass; 0: constant
 };
 
 constexpr int kFirstInit = 0x7F7F7F7F;   // memset byte 0x7F

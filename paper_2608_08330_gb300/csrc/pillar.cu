@@ -528,14 +528,18 @@ k_pfn(const PillarBufs b, const float* __restrict__ w, const float* __restrict__
   __shared__ float2 s_wb[C];
   __shared__ float4 s_pts[kPfnWarps][2][33];
   pdl_trigger();
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {      // weights: constant
+  // A context's weights are constant: they are folded while the scan runs.  The
+  // caller's own weights may be the output of the kernel before this pass, and
+  // every kernel of the pass may start before that one has ended.
+  if (b.caller_weights) pdl_wait();
+  for (int c = threadIdx.x; c < C; c += blockDim.x) {
     const float* wr = w + c * 9;
     const int wp = (c % (C / 16)) * 16 + c / (C / 16);
     s_wf[wp] = make_float4(wr[0] + wr[4] + wr[7], wr[1] + wr[5] + wr[8], wr[2] + wr[6], wr[3]);
     s_wk[wp] = make_float4(wr[0], wr[1], wr[4], wr[5]);
     s_wb[wp] = make_float2(wr[6], bias[c]);
   }
-  pdl_wait();
+  if (!b.caller_weights) pdl_wait();
   span_begin(b.pfn_span);
   __syncthreads();
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;

@@ -72,9 +72,13 @@ rtcc_status scratch_address(unsigned char** out) {
   return RTCC_OK;
 }
 
-// Programmatic on both sides, like the pass's other kernels: with full launch
-// boundaries before and after it a pass of 2048 points took 18.4 us (now 16.4),
-// one of 130000 points 24.6 us (now 23.3).
+// Programmatic on both sides, like the pass's other kernels, so calls that
+// follow each other overlap at their ends: with full launch boundaries before
+// and after it a pass of 2048 points took 18.4 us (now 16.4), one of 130000
+// points 24.6 to 25.3 us (now 24.4 to 24.6).  Nothing of a pass may then touch
+// memory before its pdl_wait, neither the shared array, which the call before
+// may still use, nor the caller's: what the caller enqueued before the call
+// may still run.
 __global__ void k_static_reset(int n, int cells, int* __restrict__ n_slot,
                                int* __restrict__ cnt_cell, int* __restrict__ first_cell,
                                int* __restrict__ stats) {
@@ -153,6 +157,7 @@ extern "C" rtcc_status rtcc_pillarise_noalloc(const rtcc_model_config* cfg, cons
   b.N = cfg->max_pts;
   b.C = cfg->pfn_ch;
   b.clear_all = 1;                              // the caller's image and cell2pillar: unknown content
+  b.caller_weights = 1;
 
   int blocks = (int)((cells + 255) / 256);
   if (blocks < 1) blocks = 1;

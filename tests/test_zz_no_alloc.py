@@ -15,9 +15,12 @@ call after the other, and requires for each:
 
 The second call also shows that leftovers of the first call in the shared
 array do not leak into the next result.  Oversized and misaligned requests
-must be refused before any work is enqueued.  The file is named to be
+must be refused before any work is enqueued.  A second test writes the weights
+on the stream directly before each call.  The file is named to be
 collected last.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -94,3 +97,44 @@ def test_noalloc_matches_oracle_and_context_on_two_calls():
                                  c2p.data_ptr(), pcell.data_ptr(), cnt.data_ptr(),
                                  stats.data_ptr(), img.data_ptr() + 8, 0)
     assert s == R.E_ARG
+
+
+@pytest.mark.parametrize("ch,points", [(32, 3000), (64, 20000)])
+def test_noalloc_reads_weights_written_just_before_it_on_the_stream(ch, points):
+    """A kernel on the same stream writes new weights directly before each of
+    many calls: every image is that of a call with the same weights long there."""
+    torch = pytest.importorskip("torch")
+    R = U.load()
+    cfg = dataclasses.replace(synth.get_config("tiny"), pfn_ch=ch, n_uniform=points, n_clusters=0)
+    c = R.model_config(cfg)
+    dev = torch.device("cuda")
+    pts = torch.from_numpy(synth.points_for(cfg, 0, 0)).to(dev)
+    cells, P = cfg.grid_w * cfg.grid_h, cfg.max_pillars
+    ints = [torch.empty(n, dtype=torch.int32, device=dev) for n in (cells, P, P, 8)]
+    # the weights are the tail of what the kernel writes, its last blocks' part
+    n_w, n_all, calls = ch * 9, 4 << 20, 40
+    rng = np.random.default_rng(ch)
+    new = torch.zeros(calls, ch * 10, device=dev)
+    new.copy_(torch.from_numpy(rng.standard_normal((calls, ch * 10)).astype(np.float32)))
+    src, dst = torch.zeros(n_all, device=dev), torch.zeros(n_all, device=dev)
+    tail = dst[n_all - ch * 10:]
+    imgs = torch.empty(2, calls, cells * ch, dtype=torch.int16, device=dev)
+
+    def call(img):
+        s = R.rtcc_pillarise_noalloc(c, pts.data_ptr(), pts.shape[0], tail.data_ptr(),
+                                     tail.data_ptr() + 4 * n_w, *[t.data_ptr() for t in ints],
+                                     img.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        assert s == R.OK, R.rtcc_status_str(s)
+
+    for i in range(calls):                             # the weights there before the call
+        tail.copy_(new[i])
+        torch.cuda.synchronize()
+        call(imgs[0, i])
+        torch.cuda.synchronize()
+    for i in range(calls):                             # written by the kernel before it
+        src[n_all - ch * 10:] = new[i]
+        torch.add(src, 0.0, out=dst)
+        call(imgs[1, i])
+    torch.cuda.synchronize()
+    assert torch.equal(imgs[0], imgs[1])
+    assert not torch.equal(imgs[0, 0], imgs[0, 1])
