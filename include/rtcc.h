@@ -367,9 +367,10 @@ rtcc_status rtcc_get_pillars(struct rtcc_ctx* ctx, int32_t agent,
  *   which = 9: fused map [H'][W'][C_feat] (agent ignored; needs
  *              RTCC_FLAG_KEEP_FUSED or attention fusion, or with
  *              RTCC_FLAG_MULTISCALE the neck's output on the fused blocks)
- *              Where the frame does not store them, 8 and 9 are computed by
- *              this call from the blocks' outputs, which stand until the next
- *              frame's first release.
+ *              It stands until the next frame's post-join; 0 to 8 of an agent
+ *              until its branch runs again.  Where a frame does not store the
+ *              neck's output (8; 9 with RTCC_FLAG_MULTISCALE), this call
+ *              computes it from the blocks' maps.
  *   which = 10..9+n_blocks: RTCC_FLAG_MULTISCALE: fused map of block
  *              which-10 [H_b][W_b][C_b] (agent ignored)
  *   which = 16 + i: output of the i-th 3x3 conv of the branch, counting

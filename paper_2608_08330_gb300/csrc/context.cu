@@ -97,8 +97,8 @@ struct rtcc_ctx {
   // fuses each block's map across the agents, then runs the neck once
   bool ms = false;
   // The post-join runs the neck, the fusion and the head in one kernel over
-  // the blocks' outputs (neck_head.cu), and the feature maps (single-scale
-  // attention: the fused map too) are computed only when they are read back
+  // the blocks' outputs (neck_head.cu), and the feature maps (multi-scale: the
+  // neck's output) are computed only when they are read back
   bool fused_neck = false;
   void* fblk[RTCC_MAX_BLOCKS] = {};   // fused block maps [H_b][W_b][C_b]
   void* neck_out = nullptr;           // neck of the fused blocks [H'][W'][C_feat]
@@ -106,7 +106,6 @@ struct rtcc_ctx {
   BackboneParams* neck_p = nullptr;
   unsigned* neck_bar = nullptr;       // [kBarWords], zero between launches
   int* d_one = nullptr;               // [RTCC_MAX_AGENTS] = {1, 0, ...}: the head's one input
-  int* d_read = nullptr;              // [RTCC_MAX_AGENTS] presence flags of a read-back's fusion
   int post_kernels = 0;               // kernels of the post-join graph
   size_t img_elems = 0, feat_elems = 0;
   std::vector<ConvLayer> layers;      // the layer list (N tiles of a one-agent launch)
@@ -156,7 +155,6 @@ struct rtcc_ctx {
   cudaEvent_t ev_post0 = nullptr, ev_fuse0 = nullptr, ev_fuse1 = nullptr, ev_post1 = nullptr;
   // frame bookkeeping
   bool post_launched = false;
-  int post_present[RTCC_MAX_AGENTS] = {};   // the agents of the last post-join
   bool closed_pending = false;
   double t_last_event = 0.0;
   rtcc_frame_info info{};
@@ -786,25 +784,6 @@ rtcc_status capture_branch(rtcc_ctx* c, int k) {
   return capture_branch_graph(c, k, ph, false, &b.pill_host);
 }
 
-// Attention over the agents' feature slots, into the context's fused map; with
-// the same bytes as the kernel that runs the neck itself where that kernel
-// takes the network.
-FuseBlocksArgs slot_attention(rtcc_ctx* c, const int* present) {
-  FuseBlocksArgs fb{};
-  fb.n = 1;
-  fb.src[0] = c->feat_all;
-  fb.cells[0] = c->Wf * c->Hf;
-  fb.ch[0] = c->Cf;
-  fb.astride[0] = (long long)c->feat_elems;
-  fb.dst[0] = c->fused;
-  fb.present = present;
-  fb.K = c->K;
-  fb.attention = 1;
-  const rtcc_model_config& g = c->cfg;
-  fb.slot_order = g.up_stride[0] != 0 && neck_head_ok(g.n_blocks, g.block_ch, g.up_stride, g.up_ch);
-  return fb;
-}
-
 rtcc_status capture_post(rtcc_ctx* c) {
   const bool tl = (c->cfg.flags & RTCC_FLAG_TIMELINE) != 0;
   // multi-scale placement: fuse each block's outputs, run the neck once on the
@@ -816,7 +795,19 @@ rtcc_status capture_post(rtcc_ctx* c) {
   const bool attn1 = !c->ms && c->cfg.fusion == RTCC_FUSE_ATTN && fuse_tc_chunk(c->Cf, 1) > 0 && c->fused;
   FuseBlocksArgs fb{};
   if (attn1) {
-    fb = slot_attention(c, c->d_present);
+    // with the same bytes as the kernel that runs the neck itself where that
+    // kernel takes the network
+    const rtcc_model_config& g = c->cfg;
+    fb.n = 1;
+    fb.src[0] = c->feat_all;
+    fb.cells[0] = c->Wf * c->Hf;
+    fb.ch[0] = c->Cf;
+    fb.astride[0] = (long long)c->feat_elems;
+    fb.dst[0] = c->fused;
+    fb.present = c->d_present;
+    fb.K = c->K;
+    fb.attention = 1;
+    fb.slot_order = g.up_stride[0] != 0 && neck_head_ok(g.n_blocks, g.block_ch, g.up_stride, g.up_ch);
     fb.span = c->fuse_span;
   } else if (c->ms) {
     fb.n = c->cfg.n_blocks;
@@ -851,6 +842,7 @@ rtcc_status capture_post(rtcc_ctx* c) {
     a.present = c->ms ? c->d_one : c->d_present;
     a.K = c->ms ? 1 : c->K;
     a.attention = !c->ms && c->cfg.fusion == RTCC_FUSE_ATTN;
+    a.fused = c->fused;
     a.head_b = c->head_b;
     a.head_out = c->head_out;
     a.keys = c->keys;
@@ -1064,14 +1056,13 @@ rtcc_status init_impl(rtcc_ctx* c, const float* weights) {
   for (int k = 0; k < c->K; ++k) fp[k] = c->br[k].feat;
   CK(cudaMemcpy(c->d_feat_ptrs, fp, sizeof(fp), cudaMemcpyHostToDevice));
   RS(dalloc(c, &c->head_out, (size_t)cells_f * 16 * sizeof(float)));
-  // attention fusion writes the fused map (the head then reads it), so it always
-  // has one; max fusion keeps it only for parity read-backs
+  // attention fusion always writes the fused map; max fusion keeps it only for
+  // parity read-backs
   if ((g.flags & RTCC_FLAG_KEEP_FUSED) || (g.fusion == RTCC_FUSE_ATTN && !c->ms))
     RS(dalloc(c, &c->fused, (size_t)cells_f * c->Cf * 2));
   {
     int one[RTCC_MAX_AGENTS] = {1};
     RS(dalloc(c, &c->d_one, sizeof(one)));
-    RS(dalloc(c, &c->d_read, sizeof(one)));
     CK(cudaMemcpy(c->d_one, one, sizeof(one), cudaMemcpyHostToDevice));
   }
   const size_t nkeys = decode_key_capacity(cells_f * g.anchors);
@@ -1278,10 +1269,8 @@ rtcc_status launch_batch(rtcc_ctx* c) {
 rtcc_status launch_post(rtcc_ctx* c) {
   // the presence flags are set on the device by the branches that ran (their
   // first kernel) and cleared by the decode kernel
-  for (int k = 0; k < c->K; ++k) {
-    c->post_present[k] = c->ctrl.present(k) ? 1 : 0;
-    if (c->post_present[k]) CK(cudaStreamWaitEvent(c->post, c->br[k].feat_ev, 0));
-  }
+  for (int k = 0; k < c->K; ++k)
+    if (c->ctrl.present(k)) CK(cudaStreamWaitEvent(c->post, c->br[k].feat_ev, 0));
   *c->h_done = 0;                                 // the decode kernel sets it when the boxes are written
   std::atomic_thread_fence(std::memory_order_seq_cst);
   CK(cudaGraphLaunch(c->post_exec, c->post));
@@ -1812,8 +1801,10 @@ rtcc_status rtcc_get_pillars(rtcc_ctx* c, int32_t agent, int32_t* host_cell2pill
 }
 
 // With the neck fused into the head's kernel no launch stores the feature
-// maps: run the deconvs of one agent (multi-scale: of the fused maps) over the
-// blocks' outputs of the last frame.  Mutex held, the branches' streams idle.
+// maps: run the deconvs of one agent over its blocks' outputs (the agent's own
+// branch is the only writer), multi-scale of the last post-join's fused maps.
+// Mutex held, the agent's stream and the batched launches' idle; other branches
+// may be running, and the deconvs wait for nothing of theirs.
 static rtcc_status run_neck(rtcc_ctx* c, int agent) {
   c->neck_p->agents[0] = c->ms ? 0 : agent;
   CK(cudaStreamSynchronize(c->post));
@@ -1836,19 +1827,7 @@ rtcc_status rtcc_get_tensor(rtcc_ctx* c, int32_t agent, int32_t which, uint16_t*
     CK(cudaStreamSynchronize(c->post));
     src = f;
     n = (size_t)c->Wf * c->Hf * c->Cf;
-    if (host_out && cap >= n && c->fused_neck) {
-      if (c->ms) {
-        RS(run_neck(c, 0));
-      } else {
-        // single-scale attention: the maps of the last post-join's agents (a
-        // new frame may have begun), then their fusion
-        for (int k = 0; k < c->K; ++k)
-          if (c->post_present[k]) RS(run_neck(c, k));
-        CK(cudaMemcpy(c->d_read, c->post_present, sizeof(c->post_present), cudaMemcpyHostToDevice));
-        CK(launch_fuse_blocks(slot_attention(c, c->d_read), c->bf16, c->post));
-        CK(cudaStreamSynchronize(c->post));
-      }
-    }
+    if (host_out && cap >= n && c->fused_neck && c->ms) RS(run_neck(c, 0));
   } else if (which >= 10 && which < 10 + c->cfg.n_blocks) {
     if (!c->ms) return RTCC_E_STATE;
     CK(cudaStreamSynchronize(c->post));

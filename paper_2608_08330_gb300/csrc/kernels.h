@@ -330,6 +330,7 @@ struct NeckHeadArgs {
   const int* present;                   // device [K]
   int K;
   int attention;                        // 0: max, 1: ego-query attention (agent 0 present)
+  void* fused;                          // attention: the fused map [H'][W'][128 n_blocks]
   const float* head_b;                  // device [16]
   float* head_out;                      // device [cells][16]
   uint32_t* keys;                       // device [cells][anchors] decode keys
@@ -344,6 +345,8 @@ struct NeckHeadParams {
   CUtensorMap in[RTCC_MAX_BLOCKS];      // 5-D view (r C, W / r, r, H / r, agent), box (64, tw, 1, th, 1)
   CUtensorMap w[RTCC_MAX_BLOCKS];       // deconv weights, box (64, 128)
   CUtensorMap wh;                       // head weights, box (64, 16)
+  CUtensorMap fused;                    // attention: 5-D view (C_feat, S, W' / S, S, H' / S) of the
+                                        // fused map, box (64, 1, tw, 1, th)
   const float* bias[RTCC_MAX_BLOCKS];
   int cin[RTCC_MAX_BLOCKS], s[RTCC_MAX_BLOCKS];
   int n_blocks, S;                      // S: the largest deconv stride

@@ -32,6 +32,10 @@
 // Storing the maps cost 68 us of deconvs in the branches' launch, 38 us of
 // fusion and 14 us of head.  Where the maps are stored all the same,
 // k_fuse_slots (fuse_blocks.cu) takes the sums in this kernel's order.
+// The fused map itself is written out: it stands for read-backs until the next
+// frame's fusion, whatever the branches have overwritten by then.  The chunks
+// the head reads go out as TMA boxes beside its MMAs, 27 MB on the 352 x 100
+// map: the frame of 5 agents takes 482 us with the store and 481 to 484 without.
 //
 // Work item: 128 cells that share their position (sy, sx) modulo the largest
 // stride S, i.e. cells (S qy + sy, S qx + sx) of a tw x th rectangle of
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_con
   uint64_t* wempty = wfull + 1;                // the MMAs that read them are done
   uint64_t* hwfull = wempty + 1;               // head weights landed
   uint64_t* fready = hwfull + 1;               // fused chunk pair written
-  uint64_t* fempty = fready + 1;               // head MMAs have read it
+  uint64_t* fempty = fready + 1;               // head MMAs (and the fused map's store) have read it
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fempty + 1);
   __shared__ __align__(16) float s_bias[RTCC_MAX_BLOCKS][kUp];
   __shared__ int s_list[RTCC_MAX_AGENTS];
@@ -167,7 +171,7 @@ __global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_con
     mbar_init(wempty, 1);
     mbar_init(hwfull, 1);
     mbar_init(fready, kEpiWarps);
-    mbar_init(fempty, 1);
+    mbar_init(fempty, ATTN ? 2 : 1);           // the head MMAs' commit; the fused map's store
     fence_barrier_init();
   }
   if (warp == kMmaWarp) {
@@ -423,9 +427,31 @@ __global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_con
 #pragma unroll
     for (int o = 0; o < kFuseHeadOut; ++o) hb[o] = P.head_b[o];
     bool alive = true;
+    uint32_t ph = 0;
     for (int t = lo; t < hi; ++t) {
       const int n = t - lo, acc = n & 1;
       const NhItem I = item_at(P, t);
+      if (ATTN && warp == kHeadWarp0) {
+        // store the item's fused chunk pairs (its boxes start inside the map;
+        // what lies beyond the map is not written)
+        for (int b = 0; b < nb; ++b, ++ph) {
+          if (alive && !mbar_wait_warp(fready, ph & 1, P.wait_budget)) {
+            if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
+            alive = false;
+          }
+          if (lane == 0) {
+            if (alive) {
+#pragma unroll
+              for (int q = 0; q < 2; ++q)
+                tma_store_5d(&P.fused, fsm + q * kChunk, b * kUp + q * 64, I.sx, I.x0, I.sy, I.y0);
+              bulk_commit();
+              bulk_wait_read_all();
+            }
+            mbar_arrive(fempty);
+          }
+          __syncwarp();
+        }
+      }
       if (alive && !mbar_wait(&hfull[acc], (n >> 1) & 1, P.wait_budget)) {
         if (lane == 0) atomicOr(P.err, ERR_WAIT_FUSE);
         alive = false;
@@ -456,6 +482,7 @@ __global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_con
         }
       }
     }
+    if (ATTN && warp == kHeadWarp0 && lane == 0) bulk_wait_all();
   } else if (warp < kMmaWarp) {
     // ---------------- TMA producers (one thread in each of 4 warps) ----------------
     if (lane == 0 && lo < hi) {
@@ -631,7 +658,7 @@ void neck_head_tile(int W, int H, int* tw, int* th) {
 
 cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P) {
   if (!neck_head_ok(a.n_blocks, a.cin, a.stride, kUp) || a.K < 1 || a.K > RTCC_MAX_AGENTS ||
-      a.anchors < 1 || a.anchors > kFuseHeadOut || a.wait_budget < 1)
+      a.anchors < 1 || a.anchors > kFuseHeadOut || a.wait_budget < 1 || (a.attention && !a.fused))
     return cudaErrorInvalidValue;
   std::memset(P, 0, sizeof(*P));
   int S = 1;
@@ -661,9 +688,16 @@ cudaError_t neck_head_fill(const NeckHeadArgs& a, bool bf16, NeckHeadParams* P) 
     e = tmap_2d(&P->w[b], a.w[b], bf16, C, (uint64_t)(s * s * kUp), 64, kUp, 128);
     if (e != cudaSuccess) return e;
   }
-  const cudaError_t e =
-      tmap_2d(&P->wh, a.head_w, bf16, (uint64_t)(a.n_blocks * kUp), kFuseHeadOut, 64, kFuseHeadOut, 128);
+  const uint64_t Cf = (uint64_t)(a.n_blocks * kUp), W = (uint64_t)a.feat_w, s64 = (uint64_t)S;
+  cudaError_t e = tmap_2d(&P->wh, a.head_w, bf16, Cf, kFuseHeadOut, 64, kFuseHeadOut, 128);
   if (e != cudaSuccess) return e;
+  if (a.attention) {
+    const uint64_t dims[5] = {Cf, s64, W / s64, s64, (uint64_t)a.feat_h / s64};
+    const uint64_t strides[4] = {Cf * 2, s64 * Cf * 2, W * Cf * 2, s64 * W * Cf * 2};
+    const uint32_t box[5] = {64, 1, (uint32_t)P->tw, 1, (uint32_t)P->th};
+    e = tmap_nd(&P->fused, a.fused, bf16, 5, dims, strides, box, 128);
+    if (e != cudaSuccess) return e;
+  }
   P->K = a.K;
   P->attention = a.attention;
   P->inv_sqrt_c = 1.0f / sqrtf((float)(a.n_blocks * kUp));

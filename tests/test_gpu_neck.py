@@ -2,12 +2,15 @@
 the head from the blocks' outputs, against the path that stores the neck's maps
 (RTCC_FLAG_KEEP_FUSED), for tiles that are ragged, single and narrow, one to
 three blocks, absent agents and both storage types: the same sums, so the same
-bytes; and the feature maps, which are then computed when they are read."""
+bytes; and the feature maps, which are then computed when they are read, and
+how long the maps stand."""
 import dataclasses
+import time
 
 import pytest
 
 import synth
+from paper_2608_08330_gb300 import rtcc as R0
 from tests import gpu_util as U
 
 pytestmark = pytest.mark.gpu
@@ -92,3 +95,36 @@ def test_neck_attention_head_matches_the_stored_maps(R, cfg, absent):
         finally:
             R.rtcc_destroy(ctx)
     assert all(g == got[0] for g in got[1:])
+
+
+@pytest.mark.parametrize("flags", [0, R0.FLAG_KEEP_FUSED], ids=["computed by the head's kernel", "stored slots"])
+def test_fused_map_stands_until_the_next_post_join(R, flags):
+    """The last frame's fused map, and the feature slots of agents that the open
+    frame has not released, while the open frame's branches overwrite their
+    blocks' outputs."""
+    cfg = _cfg(328, 184, 3, "bf16", fusion="attn")
+    old, new = ([synth.points_for(cfg, f, k) for k in range(3)] for f in (0, 1))
+    ctx, _ = U.make_ctx(cfg, flags=flags)
+    try:
+        U.run_frame(ctx, cfg, old, [0.0, 0.0, 0.0], R.MODE_RTCC)
+        fused = R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes()
+        feat0 = R.rtcc_get_tensor(ctx, 0, R.TENSOR_FEAT).tobytes()
+        block1 = R.rtcc_get_tensor(ctx, 1, 1).tobytes()
+        assert R.rtcc_frame_begin(ctx, 1, 0.0) == R.OK
+        for k in (1, 2):
+            assert R.rtcc_payload_complete(ctx, k, new[k], 0.0) == R.OK
+        end = time.monotonic() + 20                    # branch 1 has run
+        while R.rtcc_get_tensor(ctx, 1, 1).tobytes() == block1:
+            assert time.monotonic() < end
+        for _ in range(20):
+            assert R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes() == fused
+            assert R.rtcc_get_tensor(ctx, 0, R.TENSOR_FEAT).tobytes() == feat0
+        assert R.rtcc_payload_complete(ctx, 0, new[0], 1.0) == R.OK
+        s, _, _ = R.rtcc_wait_detection(ctx, 60000)
+        assert s == R.OK
+        after = R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes()
+        assert after != fused
+        U.run_frame(ctx, cfg, new, [0.0, 0.0, 0.0], R.MODE_BARRIER)
+        assert R.rtcc_get_tensor(ctx, 0, R.TENSOR_FUSED).tobytes() == after
+    finally:
+        R.rtcc_destroy(ctx)
