@@ -505,19 +505,19 @@ typedef struct {
   int32_t wide;         /* 1: tiles of 16 x 8 pixels (stride-2 and other
                            layers that load one box per tap)                */
   int32_t m_tiles;      /* pixel tiles covering one agent's output          */
-  int32_t items;        /* work items of the launch:
-                           n_batch x m_tiles x (cout / bn) x splits         */
+  int32_t items;        /* K slices of tiles in the launch:
+                           n_batch x m_tiles x (cout / bn) x splits; those
+                           of a tile are one work item where all of them do
+                           not fit a clustered grid                         */
 } rtcc_conv_plan;
 
 /*
- * The tile choice for one 3x3 conv layer (pad 1) of a backbone launch over
- * n_batch agents on `grid` CTAs whose layers wait for each other, as rtcc_init
- * makes it for n_batch = 1 (launches over several agents flow from layer to
- * layer; rtcc_init then counts items / grid, at least 1, in place of whole
- * rounds): kind 0 = stride 1,
+ * The tile choice that rtcc_init makes for one 3x3 conv layer (pad 1) of a
+ * backbone launch over n_batch agents on `grid` CTAs: kind 0 = stride 1,
  * 1 = stride 2; cin, cout its channels; out_w x out_h its output.  The K
  * slices come from the one-agent cost model, the N tile and tile shape from
- * the cost model at n_batch (rounds of items over the grid x k-blocks per
+ * the cost model at n_batch (rounds of items over the grid, whole ones for one
+ * agent, else items / grid and at least 1, x k-blocks per
  * item x the k-block's MMA time).  Pure host arithmetic: no device, no
  * context.  RTCC_E_ARG unless kind is 0 or 1, cin is a power of two in
  * 32..256, cout is a multiple of 32 in 32..256, the extents and grid are

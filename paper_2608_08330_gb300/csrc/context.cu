@@ -405,22 +405,23 @@ constexpr size_t kFrameZeroBytes = 8 * sizeof(int) + kBarWords * sizeof(unsigned
 // (halo layers without split-K: two 128-row MMAs on every weight box) costs
 // kTallCost short k-blocks per k-block -- more than one because it does
 // twice the MMAs, less than two because it halves the weight boxes per FLOP,
-// which bound a short k-block once every CTA has several items.  The tile
-// may also be laid the other way round (a halo layer's tiles transposed, a
-// tap-box layer's 16 x 8 instead of 8 x 16): the same work per item, but a
-// different item count where the image's sides are not multiples of the
-// tile's (352 x 100 in 8 x 16 tiles: 308 items, 3 rounds on 152 CTAs;
-// transposed, 286).  Ties go to the short, then the narrower tile, then the
-// first orientation.
+// which bound a short k-block once every CTA has several items.  The layers of
+// a one-agent launch wait for each other, so it takes whole rounds.  In a
+// launch over several agents the layers' items follow each other round-robin
+// without a barrier in between, so a layer's last, partly filled round costs
+// its share only (items / grid), and a layer with fewer items than CTAs an
+// item's time.  The tile may also be laid the other way round (a halo layer's
+// tiles transposed, a tap-box layer's 16 x 8 instead of 8 x 16): the same work
+// per item, but a different item count where the image's sides are not
+// multiples of the tile's (352 x 100 in 8 x 16 tiles: 308 items, 3 rounds on
+// 152 CTAs; transposed, 286).  Ties go to the short, then the narrower tile,
+// then the first orientation.  A split layer's tiles are always 64 wide: the
+// DSMEM exchange takes them, and the four slices of one stand side by side in
+// an accumulator where a CTA takes them all.
 constexpr double kTallCost = 1.6;
 double kblock_cost(int bn) { return bn >= 128 ? 1.0 : bn >= 64 ? 0.75 : 0.70; }
-//
-// `flow`: rounds are counted as items / grid, at least 1, instead of whole
-// rounds.  In a launch over several agents the layers' items follow each other
-// round-robin without a barrier between layers, so a layer's last, partly
-// filled round costs its share only; a layer with fewer items than CTAs still
-// takes an item's time.
-void pick_tile_batch(const ConvLayer L0, int sp, int grid, int batch, bool need64, bool flow, ConvLayer* out) {
+void pick_tile_batch(const ConvLayer L0, int sp, int grid, int batch, ConvLayer* out) {
+  const bool need64 = sp > 1, flow = batch > 1;
   double best = 1e30;
   out->bn = std::min(L0.cout, 64);
   out->tall = out->tr = out->wide = 0;
@@ -464,22 +465,9 @@ void choose_split(ConvLayer& L, int grid) {
 }
 
 // The N tile and tile shape of conv layer L (K slices already chosen) in a
-// launch over nb agents whose layers wait for each other.  A split layer whose
-// items fit the clustered grid keeps 64-wide tiles, which the DSMEM exchange
-// takes.
+// launch over nb agents.
 void choose_tiles(ConvLayer& L, int grid, int nb) {
-  const int m_tiles = conv_m_tiles(L);
-  const bool dsm_fit = L.splits > 1 && nb * m_tiles * (L.cout / 64) * L.splits <= grid;
-  pick_tile_batch(L, L.splits, grid, nb, dsm_fit, false, &L);
-  L.n_tiles_n = L.cout / L.bn;
-}
-
-// The tiles of the launches themselves: a one-agent launch waits layer by
-// layer, so choose_tiles; over several agents the layers flow.  A split
-// layer's tiles are always 64 wide, for the DSMEM exchange or for the four
-// slices of a tile side by side in one accumulator.
-void choose_launch_tiles(ConvLayer& L, int grid, int nb) {
-  pick_tile_batch(L, L.splits, grid, nb, L.splits > 1, nb > 1, &L);
+  pick_tile_batch(L, L.splits, grid, nb, &L);
   L.n_tiles_n = L.cout / L.bn;
 }
 
@@ -616,7 +604,7 @@ rtcc_status build_backbone(rtcc_ctx* c) {
   for (int nb = 1; nb <= K; ++nb) {
     std::vector<ConvLayer> Lb = c->layers;
     for (ConvLayer& L : Lb) {
-      if (L.kind != DECONV) choose_launch_tiles(L, grid, nb);
+      if (L.kind != DECONV) choose_tiles(L, grid, nb);
       if (conv_make_maps(L, c->bf16) != cudaSuccess) return RTCC_E_CUDA;
     }
     if (nb == 1) c->layers = Lb;                      // the maps of the one-agent tiles
