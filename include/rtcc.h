@@ -558,8 +558,8 @@ rtcc_status rtcc_test_unreachable_wait(struct rtcc_ctx* ctx);
  * *n_out.  Boxes are rectangles in x-y: centre (x, y), length l along
  * (cos yaw, sin yaw), width w across it; z, h and score are carried along.
  * Synchronous, and safe from several threads: each call takes a workspace of
- * its own (36 KB of pinned and 50 KB of device memory), of which up to four stay
- * allocated for later calls.
+ * its own (36 KB of pinned and 50 KB of device memory), of which up to four for
+ * each CUDA context stay allocated for later calls.
  */
 rtcc_status rtcc_nms(const rtcc_box* host_in, int32_t n, float iou, rtcc_box* host_out,
                      int32_t* n_out);

@@ -29,10 +29,9 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
-#include <new>
-#include <vector>
 
 #include "common.cuh"
+#include "kept_pool.h"
 #include "kernels.h"
 #include "rtcc.h"
 
@@ -351,6 +350,53 @@ cudaError_t launch_nms(const NmsArgs& a, cudaStream_t st) {
 namespace rtcc {
 namespace {
 
+// Driver calls without a runtime counterpart, looked up once; null without them.
+struct Driver {
+  CUresult (*get_current)(CUcontext*) = nullptr;
+  CUresult (*get_id)(CUcontext, unsigned long long*) = nullptr;
+  CUresult (*pointer_attribute)(void*, CUpointer_attribute, CUdeviceptr) = nullptr;
+};
+const Driver* driver() {
+  static Driver d;
+  static bool ok = false;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    auto find = [](const char* name, void** f) {
+      cudaDriverEntryPointQueryResult q;
+      return cudaGetDriverEntryPointByVersion(name, f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+             q == cudaDriverEntryPointSuccess;
+    };
+    ok = find("cuCtxGetCurrent", reinterpret_cast<void**>(&d.get_current)) &&
+         find("cuCtxGetId", reinterpret_cast<void**>(&d.get_id)) &&
+         find("cuPointerGetAttribute", reinterpret_cast<void**>(&d.pointer_attribute));
+  });
+  return ok ? &d : nullptr;
+}
+
+// Id of the current CUDA context, unique over the process's life (a device
+// reset makes a new one); 0 on failure.
+unsigned long long current_context() {
+  const Driver* d = driver();
+  if (!d) return 0;
+  CUcontext cur = nullptr;
+  unsigned long long id = 0;
+  for (int tries = 0; tries < 2; ++tries) {
+    if (d->get_current(&cur) == CUDA_SUCCESS && cur && d->get_id(cur, &id) == CUDA_SUCCESS) return id;
+    if (cudaFree(nullptr) != cudaSuccess) return 0;   // brings the device's context up
+  }
+  return 0;
+}
+
+// Id of the allocation at a device address, unique over the process's life; 0
+// where there is none.
+unsigned long long buffer_id(const void* p) {
+  const Driver* d = driver();
+  unsigned long long id = 0;
+  if (!d || d->pointer_attribute(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS)
+    return 0;
+  return id;
+}
+
 // What one call needs, sized for the longest list: a pinned block the boxes
 // go out of and the kept ones come back into, their device copy with the
 // kernel's scratch, and a stream.  Allocating these per call (cudaMalloc,
@@ -372,6 +418,7 @@ struct NmsSpace {
   static constexpr size_t kHost = kRes + sizeof(DetResultHeader) + kBoxes;
 
   unsigned long long ctx = 0;                   // the CUDA context it belongs to
+  unsigned long long buffer = 0;                // the driver's id of the device block, never given again
   cudaStream_t st = nullptr;
   uint8_t* dev = nullptr;
   uint8_t* host = nullptr;
@@ -380,7 +427,7 @@ struct NmsSpace {
     ctx = id;
     if (cudaMalloc(&dev, kMask + kMaskBytes) != cudaSuccess ||
         cudaHostAlloc(&host, kHost, cudaHostAllocDefault) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess)
+        cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess || !(buffer = buffer_id(dev)))
       return false;
     std::memset(host, 0, kHost);
     // bitmask scratch all ones (see the context's allocation)
@@ -394,82 +441,17 @@ struct NmsSpace {
     st = nullptr;
     dev = host = nullptr;
   }
+  // The context is gone when its allocation is: the address then belongs to
+  // nothing, or to another allocation (asking about it does not touch it).
+  bool gone() const { return buffer_id(dev) != buffer; }
 };
 
-// Id of the current CUDA context, unique over the process's life (a device
-// reset makes a new one); 0 on failure.
-unsigned long long current_context() {
-  using GetCurrent = CUresult (*)(CUcontext*);
-  using GetId = CUresult (*)(CUcontext, unsigned long long*);
-  static GetCurrent get_current = nullptr;
-  static GetId get_id = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void *a = nullptr, *b = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess &&
-        cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess) {
-      get_current = reinterpret_cast<GetCurrent>(a);
-      get_id = reinterpret_cast<GetId>(b);
-    }
-  });
-  if (!get_current) return 0;
-  CUcontext cur = nullptr;
-  unsigned long long id = 0;
-  for (int tries = 0; tries < 2; ++tries) {
-    if (get_current(&cur) == CUDA_SUCCESS && cur && get_id(cur, &id) == CUDA_SUCCESS) return id;
-    if (cudaFree(nullptr) != cudaSuccess) return 0;   // brings the device's context up
-  }
-  return 0;
-}
-
-// Idle workspaces of earlier calls, a few at most.  A call takes one for
-// itself, so calls from several threads never share one; what does not fit on
-// return is freed.  One that belongs to a context that no longer exists went
-// with it and is only dropped.
-class NmsPool {
- public:
-  std::unique_ptr<NmsSpace> take(unsigned long long ctx) {
-    {
-      std::lock_guard<std::mutex> lk(mu_);
-      for (size_t i = idle_.size(); i-- > 0;)
-        if (idle_[i]->ctx == ctx) {
-          std::unique_ptr<NmsSpace> s = std::move(idle_[i]);
-          idle_.erase(idle_.begin() + (long)i);
-          return s;
-        }
-    }
-    std::unique_ptr<NmsSpace> s(new (std::nothrow) NmsSpace);
-    if (s && !s->create(ctx)) {
-      s->destroy();
-      s.reset();
-    }
-    return s;
-  }
-  void give(std::unique_ptr<NmsSpace> s) {
-    {
-      std::lock_guard<std::mutex> lk(mu_);
-      if (idle_.size() < kIdle) {
-        idle_.push_back(std::move(s));          // within the reserved capacity
-        return;
-      }
-    }
-    s->destroy();
-  }
-  NmsPool() { idle_.reserve(kIdle); }
-
- private:
-  static constexpr size_t kIdle = 4;            // 36 KB pinned and 50 KB device memory each
-  std::mutex mu_;
-  std::vector<std::unique_ptr<NmsSpace>> idle_;
-};
+using NmsPool = KeptPool<NmsSpace, 4>;         // 36 KB pinned and 50 KB device memory each
 // never destroyed: the driver may already be gone when the process's static
 // objects are, and it takes the workspaces with it
-NmsPool& nms_pool() {
-  static NmsPool* p = new NmsPool;
-  return *p;
+NmsPool* nms_pool() {
+  static NmsPool* p = new (std::nothrow) NmsPool;
+  return p;
 }
 
 // The kernel on n boxes with workspace s; false on a CUDA error.
@@ -522,14 +504,15 @@ extern "C" rtcc_status rtcc_nms(const rtcc_box* host_in, int32_t n, float iou, r
     return RTCC_E_ARG;
   const unsigned long long ctx = current_context();
   if (!ctx) return RTCC_E_CUDA;
-  std::unique_ptr<NmsSpace> s = nms_pool().take(ctx);
+  NmsPool* pool = nms_pool();
+  std::unique_ptr<NmsSpace> s = pool ? pool->take(ctx) : nullptr;
   if (!s) return RTCC_E_NOMEM;
   // Refused while this thread is in a stream capture that forbids unsafe calls
   // (the query is one, as an allocation is); an idle workspace's stream has
   // nothing in flight.
   const cudaError_t q = cudaStreamQuery(s->st);
   if (q != cudaSuccess && q != cudaErrorNotReady) {
-    nms_pool().give(std::move(s));
+    pool->give(std::move(s));
     return RTCC_E_CUDA;
   }
   if (!nms_on(*s, host_in, n, iou, host_out, n_out)) {
@@ -537,6 +520,6 @@ extern "C" rtcc_status rtcc_nms(const rtcc_box* host_in, int32_t n, float iou, r
     s->destroy();
     return RTCC_E_CUDA;
   }
-  nms_pool().give(std::move(s));
+  pool->give(std::move(s));
   return RTCC_OK;
 }

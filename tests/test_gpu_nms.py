@@ -4,6 +4,9 @@ list (512), duplicates, disjoint sets, suppression chains, and thresholds 0
 and 1."""
 import concurrent.futures as cf
 import math
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -92,3 +95,40 @@ def test_nms_suppressors_in_any_earlier_chunk(R, n):
     b = _boxes(np.column_stack([x, np.zeros(n), np.full(n, 4.0), np.full(n, 1.8), np.zeros(n)]))
     kept = U.check_nms(b, R.rtcc_nms(b, 0.2), 0.2)
     assert n // 4 <= len(kept) <= n // 2 + 1           # IoU 0.40 to a neighbour, 0.08 two on
+
+
+CONTEXTS = """
+import ctypes as C, sys
+import numpy as np
+from tests import gpu_util as U
+from tests.test_gpu_nms import _crowd
+R, cu = U.load(), C.CDLL("libcuda.so.1")
+boxes = [_crowd(n, n) for n in (512, 33)]
+dev, primary, cur = C.c_int(), C.c_void_p(), C.c_void_p()
+def ok(r): assert r == 0, r
+ok(cu.cuInit(0)); ok(cu.cuDeviceGet(C.byref(dev), 0)); ok(cu.cuDevicePrimaryCtxRetain(C.byref(primary), dev))
+want = None
+for turn in range(6):                       # a context of its own, then the primary one
+    ctx = C.c_void_p()
+    ok(cu.cuCtxCreate_v2(C.byref(ctx), C.c_uint(0), dev))
+    for c in (ctx, primary, ctx):
+        ok(cu.cuCtxSetCurrent(c))
+        got = [R.rtcc_nms(b, 0.2).tobytes() for b in boxes]
+        want = want or got
+        assert got == want
+        ok(cu.cuCtxGetCurrent(C.byref(cur)))
+        assert cur.value == c.value
+    ok(cu.cuCtxSetCurrent(primary))
+    ok(cu.cuCtxDestroy_v2(ctx))
+for b, g in zip(boxes, want):
+    U.check_nms(b, R.rtcc_nms(b, 0.2), 0.2)
+print("contexts ok")
+"""
+
+
+def test_nms_in_contexts_that_come_and_go(R):
+    """Calls in driver contexts that are created and destroyed, and in the primary
+    one between them: workspaces of a context that is gone are never used."""
+    r = subprocess.run([sys.executable, "-c", CONTEXTS], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "contexts ok" in r.stdout, r.stdout + r.stderr
