@@ -22,6 +22,7 @@
 //               threads, so every thread holds the same s_k; the softmax is
 //               taken online in one pass over the agents)
 // Every reduction has a fixed order: the result is bit-reproducible.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -206,98 +207,160 @@ __global__ void __launch_bounds__(kThreads, (ATTN || WIDE) ? 3 : 5) k_fuse_block
   }
 }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Attention over feature slots of C = 128 nb channels with every sum in the
 // order of the kernel that fuses without stored slots (k_neck_head), so that
 // both give the same bytes: the dot product as one chain over each 32
 // channels, those of the same 32 columns added over the nb blocks, then over
 // the four column groups; the softmax over all scores, the weights normalised
 // before the sums.  Half a warp per cell, 4 nb of its lanes own 32 channels
-// each; the maps are read twice.
+// each.  The sums need every score first, so a warp brings its two cells'
+// vectors of all agents into its part of shared memory (coalesced 16-byte
+// copies, all agents in flight together) and reads them there twice: the maps
+// are read once.  The chains' results meet in shared memory too, where one lane
+// per agent adds them and takes the agent's weight: with every lane doing so for
+// all agents the kernel was bound by instructions (2485 a warp and task; 60 us
+// for 5 agents on the 352 x 100 map).  Now, with 2, 5 and 8 agents: 22, 36 and
+// 53 us, 3.7 to 4.6 TB/s; reading the maps twice took 25, 57 and 89 us, the
+// online softmax of k_fuse_blocks, whose sums differ, takes 16, 38 and 57.
+constexpr int kDotStride = 33;                   // words per agent of a warp's 32 chain results (bank spread)
+constexpr size_t slots_warp_bytes(int K, int C) {
+  return (size_t)K * 2 * C * 2 + (size_t)(RTCC_MAX_AGENTS * kDotStride + 8) / 4 * 16;
+}
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 3) k_fuse_slots(const __grid_constant__ FuseBlocksArgs a) {
+  extern __shared__ __align__(16) uint8_t slots_smem[];
   pdl_trigger();
   pdl_wait();
   span_begin(a.span);
   unsigned pres = 0;
   for (int k = 0; k < a.K; ++k) pres |= (a.present[k] ? 1u : 0u) << k;
   const int lane = threadIdx.x & 31, h0 = lane & 16, hl = lane & 15;
-  const int C = a.ch[0], nb = C / 128;
+  const int C = a.ch[0], nb = C / 128, cpc = 16 * nb;        // 16-byte pieces per cell
   const bool mine = hl < 4 * nb;
+  const int pair = 2 * cpc;                                  // and per two cells
+  uint8_t* const wbase = slots_smem + (threadIdx.x >> 5) * slots_warp_bytes(a.K, C);
+  uint4* const ws = reinterpret_cast<uint4*>(wbase);
+  float* const dots = reinterpret_cast<float*>(ws + a.K * pair);
+  // piece v of this lane's 64 bytes: the pieces of a lane rotate with it, so
+  // that eight lanes' reads of piece v fall into different banks
+  const uint4* const rd = ws + (lane >> 4) * cpc + (mine ? hl : 0) * 4;
+  const int rot = (mine ? hl : 0) >> 1;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < a.tasks[0]; w += warps) {
-    const int cell = (int)(2 * w) + (lane >> 4);
-    const bool valid = cell < a.cells[0];
-    const size_t off = (size_t)(valid ? cell : a.cells[0] - 1) * C + (size_t)(mine ? hl : 0) * 32;
-    const T* src = static_cast<const T*>(a.src[0]) + off;
-    auto load = [&](int k, uint32_t (&x)[16]) {
+    for (int i = 0; i < nb; ++i) {
+      const int q = lane + 32 * i, c = q >= cpc ? 1 : 0, r = q - c * cpc;
+      const int row = min((int)(2 * w) + c, a.cells[0] - 1);   // past the end: the last cell, not stored
+      const T* src = static_cast<const T*>(a.src[0]) + (size_t)row * C + r * 8;
+      uint4* dst = ws + c * cpc + (r & ~3) + ((r + (r >> 3)) & 3);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const uint4 r = ld16(src + (size_t)k * a.astride[0] + 8 * v);
-        x[4 * v] = r.x;
-        x[4 * v + 1] = r.y;
-        x[4 * v + 2] = r.z;
-        x[4 * v + 3] = r.w;
+      for (int k = 0; k < RTCC_MAX_AGENTS; ++k)
+        if ((pres >> k) & 1u) cp_async16(dst + k * pair, src + (size_t)k * a.astride[0]);
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    float ego[32];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const uint4 x = rd[(v + rot) & 3];
+      const uint32_t xk[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 y = Store<T>::unpack2(xk[i]);
+        ego[8 * v + 2 * i] = y.x;
+        ego[8 * v + 2 * i + 1] = y.y;
       }
-    };
-    uint32_t q[16];
-    load(0, q);
-    float s[RTCC_MAX_AGENTS], m = -INFINITY, den = 0.f;
-#pragma unroll
-    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) {
-      if (!((pres >> k) & 1u)) continue;
-      uint32_t x[16];
-      load(k, x);
+    }
+    for (unsigned left = pres; left; left &= left - 1u) {
+      const int k = __ffs(left) - 1;
       float d = 0.f;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float2 u = Store<T>::unpack2(q[i]), v = Store<T>::unpack2(x[i]);
-        d = fmaf(u.x, v.x, d);
-        d = fmaf(u.y, v.y, d);
+      for (int v = 0; v < 4; ++v) {
+        const uint4 x = rd[k * pair + ((v + rot) & 3)];
+        const uint32_t xk[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 y = Store<T>::unpack2(xk[i]);
+          d = fmaf(ego[8 * v + 2 * i], y.x, d);
+          d = fmaf(ego[8 * v + 2 * i + 1], y.y, d);
+        }
       }
+      dots[k * kDotStride + lane] = d;
+    }
+    __syncwarp();
+    // lane hl of a cell: agent hl's score, softmax term and weight
+    const bool has = hl < RTCC_MAX_AGENTS && ((pres >> hl) & 1u);
+    float sc = -INFINITY;
+    if (has) {
+      const float* d = dots + hl * kDotStride + h0;
       float part[4];
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
-        part[g] = __shfl_sync(kFull, d, h0 + g);
-        for (int b = 1; b < nb; ++b) part[g] += __shfl_sync(kFull, d, h0 + 4 * b + g);
+        part[g] = d[g];
+        for (int b = 1; b < nb; ++b) part[g] += d[4 * b + g];
       }
-      s[k] = __fmul_rn(part[0] + part[1] + part[2] + part[3], a.inv_sqrt_c[0]);
-      m = fmaxf(m, s[k]);
+      sc = __fmul_rn(part[0] + part[1] + part[2] + part[3], a.inv_sqrt_c[0]);
     }
+    float m = sc;
 #pragma unroll
-    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) {
-      if (!((pres >> k) & 1u)) continue;
-      s[k] = expf(s[k] - m);
-      den += s[k];
-    }
-    const float inv = 1.f / den;
+    for (int o = RTCC_MAX_AGENTS / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+    const float ex = has ? expf(sc - m) : 0.f;
+    float den = 0.f;
+#pragma unroll
+    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) den += __shfl_sync(kFull, ex, h0 + k);
+    const float wgt = __fmul_rn(ex, 1.f / den);
     float f[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) f[i] = 0.f;
+    for (unsigned left = pres; left; left &= left - 1u) {
+      const int k = __ffs(left) - 1;
+      const float wk = __shfl_sync(kFull, wgt, h0 + k);
 #pragma unroll
-    for (int k = 0; k < RTCC_MAX_AGENTS; ++k) {
-      if (!((pres >> k) & 1u)) continue;
-      const float wk = __fmul_rn(s[k], inv);
-      uint32_t x[16];
-      load(k, x);
+      for (int v = 0; v < 4; ++v) {
+        const uint4 x = rd[k * pair + ((v + rot) & 3)];
+        const uint32_t xk[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float2 v = Store<T>::unpack2(x[i]);
-        f[2 * i] = fmaf(wk, v.x, f[2 * i]);
-        f[2 * i + 1] = fmaf(wk, v.y, f[2 * i + 1]);
+        for (int i = 0; i < 4; ++i) {
+          const float2 y = Store<T>::unpack2(xk[i]);
+          f[8 * v + 2 * i] = fmaf(wk, y.x, f[8 * v + 2 * i]);
+          f[8 * v + 2 * i + 1] = fmaf(wk, y.y, f[8 * v + 2 * i + 1]);
+        }
       }
     }
-    if (valid && mine) {
-      uint4* out = reinterpret_cast<uint4*>(static_cast<T*>(a.dst[0]) + off);
+    const int cell = (int)(2 * w) + (lane >> 4);
+    if (mine && cell < a.cells[0]) {
+      uint4* out = reinterpret_cast<uint4*>(static_cast<T*>(a.dst[0]) + (size_t)cell * C + hl * 32);
 #pragma unroll
       for (int v = 0; v < 4; ++v)
         out[v] = make_uint4(Store<T>::pack2(f[8 * v], f[8 * v + 1]), Store<T>::pack2(f[8 * v + 2], f[8 * v + 3]),
                             Store<T>::pack2(f[8 * v + 4], f[8 * v + 5]), Store<T>::pack2(f[8 * v + 6], f[8 * v + 7]));
     }
+    __syncwarp();                                // the next cells overwrite these
   }
   if (a.span) {
     __syncthreads();
     span_end(a.span);
   }
+}
+
+template <typename T>
+cudaError_t launch_fuse_slots(const FuseBlocksArgs& a, int sms, cudaStream_t st) {
+  constexpr int warps = kThreads / 32;
+  static_assert(slots_warp_bytes(RTCC_MAX_AGENTS, 384) * warps <= 227 * 1024, "shared memory of a block");
+  const size_t smem = slots_warp_bytes(a.K, a.ch[0]) * warps;   // 109 KB for 8 agents of 384 channels
+  const cudaError_t e = cudaFuncSetAttribute(k_fuse_slots<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(slots_warp_bytes(RTCC_MAX_AGENTS, 384) * warps));
+  if (e != cudaSuccess) return e;
+  int per = 0;                                     // one wave: a block more than fits would start at the end
+  const cudaError_t eo = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_fuse_slots<T>, kThreads, smem);
+  if (eo != cudaSuccess) return eo;
+  const long long blocks = std::min<long long>((a.tasks[0] + warps - 1) / warps, (long long)per * sms);
+  if (blocks < 1) return cudaErrorInvalidValue;
+  return launch_pdl(k_fuse_slots<T>, dim3((unsigned)blocks), dim3(kThreads), smem, st, a);
 }
 
 }  // namespace
@@ -331,9 +394,7 @@ cudaError_t launch_fuse_blocks(FuseBlocksArgs a, bool bf16, cudaStream_t st) {
   if (blocks > 8LL * sms) blocks = 8LL * sms;       // grid-stride beyond 8 blocks per SM
   if (blocks < 1) blocks = 1;
   const dim3 g((unsigned)blocks), t(kThreads);
-  if (a.slot_order)
-    return bf16 ? launch_pdl(k_fuse_slots<__nv_bfloat16>, g, t, 0, st, a)
-                : launch_pdl(k_fuse_slots<__half>, g, t, 0, st, a);
+  if (a.slot_order) return bf16 ? launch_fuse_slots<__nv_bfloat16>(a, sms, st) : launch_fuse_slots<__half>(a, sms, st);
   if (bf16) {
     if (wide)
       return a.attention ? launch_pdl(k_fuse_blocks<__nv_bfloat16, true, true>, g, t, 0, st, a)

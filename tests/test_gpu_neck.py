@@ -72,6 +72,7 @@ ATTN = [
     ("one block", _cfg(40, 24, 3, blocks=((2, 128, 2),), ups=(1,), fusion="attn"), ()),
     ("two blocks, strides 2 and 4", _cfg(48, 40, 2, "bf16", blocks=((1, 64, 1), (1, 256, 2)), ups=(1, 2),
                                          fusion="attn"), ()),
+    ("an odd number of cells", _cfg(42, 22, 5, "bf16", blocks=((1, 128, 2),), ups=(1,), fusion="attn"), (2,)),
 ]
 
 
