@@ -177,7 +177,12 @@ typedef struct {
   double t_release_ms[RTCC_MAX_AGENTS];   /* host time each branch launched   */
   float gpu_backbone_ms[RTCC_MAX_AGENTS]; /* conv/deconv span per branch; -1
                                              without RTCC_FLAG_TIMELINE        */
-  float gpu_branch_ms[RTCC_MAX_AGENTS];   /* whole branch incl. pillarise     */
+  float gpu_branch_ms[RTCC_MAX_AGENTS];   /* whole branch incl. pillarise (and
+                                             with RTCC_FLAG_NO_BATCH the wait
+                                             for another's running backbone);
+                                             -1 if its backbone came after the
+                                             release hold or in a batch, and
+                                             without RTCC_FLAG_TIMELINE        */
   float gpu_fusion_ms;              /* fusion+head kernel                     */
   float gpu_post_ms;                /* whole post-join graph                  */
   int32_t dispatch_order[RTCC_MAX_AGENTS];  /* agents in launch order, -1 pad */

@@ -58,7 +58,8 @@ struct Branch {
   cudaEvent_t feat_ev = nullptr;   // this frame: the event after which the slot is written
   int stamp_src = -1;              // this frame: whose stamps buffer its launch wrote
   int launch_idx = -1;             // this frame: index of the backbone launch that ran it
-  bool full_graph = false;         // this frame: ran as its own branch graph (event nodes)
+  bool own_launch = false;         // this frame: ran by itself from its first kernel on
+                                   // (ev_start and ev_end are this frame's)
   const float* pend_ptr = nullptr;
   int pend_n = 0;
   bool pend_resident = false;
@@ -1186,17 +1187,19 @@ rtcc_status launch_full(rtcc_ctx* c, int k) {
   b.feat_ev = b.done;
   b.stamp_src = k;
   b.launch_idx = c->n_launches;
-  b.full_graph = true;
+  b.own_launch = true;
   note_launch(c, k, 1, b.done);
   note_dispatch(c, k);
   return RTCC_OK;
 }
 
-// Branch k's pillar chain alone; its backbone joins a batch.
-rtcc_status launch_pill(rtcc_ctx* c, int k) {
+// Branch k's pillar chain alone; its backbone joins a batch, or (own) follows
+// as a launch of its own.
+rtcc_status launch_pill(rtcc_ctx* c, int k, bool own = false) {
   Branch& b = c->br[k];
   bool hv = false;
   RS(stage_payload(c, k, &hv));
+  if (own && (c->cfg.flags & RTCC_FLAG_TIMELINE)) CK(cudaEventRecord(b.ev_start, b.st));
   CK(cudaGraphLaunch(hv ? b.pill_host : b.pill, b.st));
   CK(cudaEventRecord(b.pill_done, b.st));
   c->pending.push_back(k);
@@ -1223,6 +1226,7 @@ rtcc_status launch_batch(rtcc_ctx* c) {
     if (tl) CK(cudaEventRecord(b.ev_bb0, b.st));
     CK(launch_backbone(*b.bb, c->bf16, b.st));
     if (tl) CK(cudaEventRecord(b.ev_bb1, b.st));
+    if (tl) CK(cudaEventRecord(b.ev_end, b.st));
     CK(cudaEventRecord(b.done, b.st));
     b.feat_ev = b.done;
     b.stamp_src = ag[0];
@@ -1288,8 +1292,10 @@ rtcc_status after_event(rtcc_ctx* c, const std::vector<int>& released, double t_
   if (!batching) {
     for (int k : released) {
       if (backbone_busy(c)) {
-        RS(launch_pill(c, k));
+        // its span then includes the wait for the running backbone
+        RS(launch_pill(c, k, true));
         RS(launch_batch(c));
+        c->br[k].own_launch = true;
       } else {
         RS(launch_full(c, k));
       }
@@ -1463,7 +1469,7 @@ rtcc_status rtcc_frame_begin(rtcc_ctx* c, uint64_t frame_id, double t0_ms) {
     c->br[k].feat_ev = nullptr;
     c->br[k].stamp_src = -1;
     c->br[k].launch_idx = -1;
-    c->br[k].full_graph = false;
+    c->br[k].own_launch = false;
   }
   c->info.gpu_fusion_ms = -1.f;
   c->info.gpu_post_ms = -1.f;
@@ -1591,7 +1597,7 @@ rtcc_status rtcc_wait_detection(rtcc_ctx* c, int32_t timeout_ms, rtcc_box* out, 
       float ms = -1.f;
       if (b.launch_idx >= 0 && b.launch_idx < RTCC_MAX_AGENTS)
         c->info.gpu_backbone_ms[k] = c->info.gpu_launch_ms[b.launch_idx];
-      if (b.full_graph && cudaEventElapsedTime(&ms, b.ev_start, b.ev_end) == cudaSuccess)
+      if (b.own_launch && cudaEventElapsedTime(&ms, b.ev_start, b.ev_end) == cudaSuccess)
         c->info.gpu_branch_ms[k] = ms;
       unsigned long long ps[2] = {0ull, 0ull};
       if (b.pb.pfn_span && cudaMemcpy(ps, b.pb.pfn_span, sizeof(ps), cudaMemcpyDeviceToHost) == cudaSuccess &&

@@ -50,3 +50,20 @@ def test_batched_exchanges_keep_their_agents_apart(R, w, h, agents, dtype):
             R.rtcc_destroy(ctx)
         want = want or got[0]
         assert all(g == want for g in got)
+
+
+def test_unbatched_branches_report_their_spans(R):
+    """RTCC_FLAG_NO_BATCH: a branch released while another's backbone runs waits
+    for it, and still reports its whole span."""
+    cfg = _cfg(328, 184, 4, "fp16")
+    pts = [synth.points_for(cfg, 0, k) for k in range(4)]
+    ctx, _ = U.make_ctx(cfg, flags=R.FLAG_NO_BATCH | R.FLAG_TIMELINE)
+    try:
+        for mode in (R.MODE_BARRIER, R.MODE_RTCC):
+            for f in range(5):
+                U.run_frame(ctx, cfg, pts, [0.0] * 4, mode, frame_id=f)
+                info = R.rtcc_get_frame_info(ctx)
+                for k in range(4):
+                    assert 0 < info.gpu_backbone_ms[k] < info.gpu_branch_ms[k] < 100
+    finally:
+        R.rtcc_destroy(ctx)
