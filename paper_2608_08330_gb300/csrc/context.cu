@@ -395,6 +395,7 @@ void pick_tile(int m_tiles, int co, int total_kb, int grid, int* bn_out, int* sp
 }
 
 constexpr size_t kFrameZeroBytes = 8 * sizeof(int) + kBarWords * sizeof(unsigned);
+static_assert(kFrameZeroBytes / sizeof(int) <= kCellsThreads, "cleared by one block of the first pillar kernel");
 
 // Tile of a conv layer in a launch over `batch` agents, with its K slices
 // fixed (they decide the fp32 summation order, so they are the same for every

@@ -90,6 +90,9 @@ struct PillarBufs {
 };
 
 constexpr int kFirstInit = 0x7F7F7F7F;   // memset byte 0x7F
+// A thread of the first kernel clears at most one of the n_zero words, and its
+// smallest grid is one block of this many threads.
+constexpr int kCellsThreads = 256;
 // The scan takes tiles of 4 points per thread, 256 to 1024 threads.
 constexpr int kScanTileMin = 1024;
 constexpr int kAggStride = 16;           // words between two tiles' aggregates (one line each)

@@ -83,7 +83,7 @@ __device__ __forceinline__ int2 unpack_agg(unsigned long long w) {
 }
 
 template <int CH>
-__global__ void __launch_bounds__(256) k_pillar_cells(const PillarBufs b, const GridGeom g,
+__global__ void __launch_bounds__(kCellsThreads) k_pillar_cells(const PillarBufs b, const GridGeom g,
                                                       int ntiles) {
   __shared__ int s_n;
   pdl_trigger();
@@ -672,12 +672,12 @@ cudaError_t launch_all(const PillarBufs& b, const GridGeom& g0, const float* pfn
   g.qxy_inv = 1.f / g.qxy;                                                // exact: powers of two
   g.qz_inv = 1.f / g.qz;
   const int sms = sm_count();
-  if (sms < 1 || b.stats != b.zero_words || b.n_zero < 8) return cudaErrorInvalidValue;
+  if (sms < 1 || b.stats != b.zero_words || b.n_zero < 8 || b.n_zero > kCellsThreads) return cudaErrorInvalidValue;
   constexpr int CH = C * 2 / 16;                  // 16-byte chunks per cell
   const int ntiles_max = scan_tiles(b.cap);       // the tile words the first kernel clears
   const int cells_threads = b.cap > ntiles_max ? b.cap : ntiles_max;
-  cudaError_t e = launch_pdl(k_pillar_cells<CH>, dim3((cells_threads + 255) / 256), dim3(256), 0,
-                             st, b, g, ntiles_max);
+  cudaError_t e = launch_pdl(k_pillar_cells<CH>, dim3((cells_threads + kCellsThreads - 1) / kCellsThreads),
+                             dim3(kCellsThreads), 0, st, b, g, ntiles_max);
   if (e != cudaSuccess) return e;
   // the scan: the smallest block (a multiple of 32 threads, at least 256)
   // whose tiles fit one block per SM (two scan blocks on one SM delay each
