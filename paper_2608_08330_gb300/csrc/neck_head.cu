@@ -96,7 +96,12 @@ constexpr int kFOff = kWOff + kMaxChunks * kChunk;
 constexpr int kHOff = kFOff + 2 * kChunk;
 constexpr int kBarOff = kHOff + RTCC_MAX_BLOCKS * 2 * kHeadChunk;
 constexpr int kSmem = kBarOff + 256 + 1024;    // barriers; alignment to 1024
-static_assert(kSmem <= 227 * 1024 - 2048, "shared memory budget (with the static arrays)");
+// the static arrays: biases, agent list and count, attention's weights
+constexpr int static_smem(bool attn) {
+  return RTCC_MAX_BLOCKS * kUp * 4 + RTCC_MAX_AGENTS * 4 + 16 + (attn ? RTCC_MAX_AGENTS * kTile : 1) * 4;
+}
+static_assert(kSmem + static_smem(true) <= 227 * 1024 && kSmem + static_smem(false) <= 227 * 1024,
+              "shared memory of a block");
 // the producers take turns on the stages: a thread's wait for a stage rules out
 // the phase before the one its next wait is for
 static_assert(producers(false) <= kStages, "phase parity");
@@ -146,6 +151,7 @@ __global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_con
   __shared__ int s_list[RTCC_MAX_AGENTS];
   __shared__ int s_kp;
   __shared__ float s_w[ATTN ? RTCC_MAX_AGENTS : 1][ATTN ? kTile : 1];   // an item's weights, agents in list order
+  static_assert(sizeof(s_bias) + sizeof(s_list) + sizeof(s_kp) + sizeof(s_w) <= static_smem(ATTN), "see static_smem");
 
   const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
   const int lane = threadIdx.x & 31;
