@@ -216,6 +216,10 @@ typedef struct {
  * the K branch graphs plus the post-join graph, and (unless
  * RTCC_FLAG_NO_BATCH) starts one host thread, the dispatcher of batched
  * backbone launches (see rtcc_payload_complete), which rtcc_destroy joins.
+ * Run the frames of one context at a time on a GPU: a backbone needs all of its
+ * blocks resident, a context starts one only behind its others, but nothing
+ * orders those of two contexts, and two that each hold part of the SMs wait
+ * until the limit of their waits (RTCC_E_DEVICE).
  * RTCC_E_ARG for an unsupported config or a blob of the wrong length.  A
  * grid whose x or y bounds (x_min, x_min + grid_w * pillar, and the same in
  * y) lie more than 2^20 pillar edges from 0, or whose z bounds lie more than

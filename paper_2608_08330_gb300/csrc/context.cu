@@ -1168,8 +1168,10 @@ bool backbone_busy(const rtcc_ctx* c) { return c->inflight >= 0 && c->done_words
 
 // Two backbones must never share the GPU: each needs all of its CTAs resident
 // (they wait for each other's items), and two that each hold part of the SMs
-// would wait until their bound.  A backbone launched while another runs goes
-// behind that one's event, whatever their streams.
+// would wait until their bound.  A backbone launched while another of this
+// context runs goes behind that one's event, whatever their streams.  Nothing
+// orders the backbones of two contexts: frames of theirs that overlap on one
+// GPU can still run a wait out (RTCC_E_DEVICE).
 rtcc_status after_running_backbone(rtcc_ctx* c, cudaStream_t st) {
   if (backbone_busy(c)) CK(cudaStreamWaitEvent(st, c->bb_ev, 0));
   return RTCC_OK;

@@ -24,12 +24,13 @@
 // reads has been counted.  In a launch over several agents the other agents'
 // items lie in between, so a CTA flows from one layer into the next without
 // waiting for the slowest item of all agents; a one-agent launch waits layer
-// by layer.  Keeping the CTAs resident replaces sixteen kernel boundaries (each
+// by layer, and so does a layer whose K slices meet in distributed shared
+// memory (for all agents: its receive buffers have to be free).  Keeping the CTAs resident replaces sixteen kernel boundaries (each
 // a full drain and relaunch) by counter waits, and lets the TMA/MMA pipeline
 // and the tensor-memory allocation carry across tiles and layers.
 //
 // Roles (256 threads): warps 0, 6, 7 = TMA producers, warp 1 = tensor-memory
-// owner and MMA issuer, warps 2..5 = epilogue.  Tensor memory holds two 128-column
+// owner and MMA issuer, warps 2..5 = epilogue.  Tensor memory holds two 256-column
 // accumulators, so the epilogue of one tile overlaps the MMAs of the next.
 // The epilogue adds bias, applies ReLU, rounds to 16 bits and writes each
 // pixel's channels from registers (16-byte stores; an item's stores are then
@@ -37,9 +38,8 @@
 // in slice order, on four CTAs through distributed shared memory or, where the
 // items of a launch do not fit the clustered grid, on one CTA in four
 // accumulators side by side: the same sums, and results do not depend on
-// timing.  Every
-// wait is bounded; one that runs out sets a bit in the error word and the CTA
-// winds down instead of hanging.
+// timing.  Every wait is bounded; one that runs out sets a bit in the error
+// word and the CTA winds down instead of hanging.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -419,8 +419,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_backbone(const __grid_constant_
   const int lane = threadIdx.x & 31;
   // The DSMEM reduction needs the launch to be in clusters of kMaxSplits CTAs;
   // the cluster size is read from the hardware, not trusted from the
-  // parameters, and without such clusters split layers reduce through global
-  // memory (the workspace exists for every split layer).
+  // parameters, and without such clusters one CTA accumulates all slices of a
+  // tile side by side in tensor memory.
   const uint32_t ncl = cluster_nctarank();
   const bool clustered = ncl == (uint32_t)kMaxSplits;
 

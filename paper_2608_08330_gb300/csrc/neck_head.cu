@@ -59,8 +59,10 @@
 // (tensor-memory lane quarter warp % 4, columns 32 (warp / 4)), warps 16..19
 // head epilogue, then four warps (attention three) with one TMA producer thread
 // each (a thread's boxes complete one after another, so the stages are dealt
-// over them), the last warp tensor-memory owner and MMA issuer.  Every wait is bounded (an error bit, no hang); the summation order
-// is fixed, so the output is bit-reproducible.
+// over them), the last warp tensor-memory owner and MMA issuer.  Attention's
+// first head epilogue warp also stores the fused map.  Every wait is bounded (an
+// error bit, no hang); the summation order is fixed, so the output is
+// bit-reproducible.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(threads(ATTN), 1) k_neck_head(const __grid_con
     }
     if (ATTN && warp == kHeadWarp0 && lane == 0) bulk_wait_all();
   } else if (warp < kMmaWarp) {
-    // ---------------- TMA producers (one thread in each of 4 warps) ----------------
+    // ---------------- TMA producers (one thread in each of kProducers warps) ----------------
     if (lane == 0 && lo < hi) {
       const uint32_t bytes = (uint32_t)(P.tw * P.th * 128);
       uint32_t it = 0, loads = 1, mine = 0;    // weight loads so far; this thread's last stage + 1

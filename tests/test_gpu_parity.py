@@ -342,8 +342,8 @@ def test_decode_level1_list_path(R):
 
 def test_split_k_without_clusters_bit_identical(R):
     # The deepest block's 4-way split-K reduces through distributed shared
-    # memory when the backbone runs in clusters of four CTAs, and through
-    # global memory without clusters; both sum the slices in slice order, so
+    # memory when the backbone runs in clusters of four CTAs; without clusters
+    # one CTA accumulates the slices side by side.  Both sum them in order, so
     # the outputs must match bit for bit (and the oracle within tolerance).
     cfg = _small_pp()
     pts = [synth.points_for(cfg, 0, k) for k in range(cfg.n_agents)]
